@@ -207,11 +207,14 @@ LBMRV_API int lbmrv_init_equilibrium(lbmrv_t h, const float* rho_dev, const floa
  * reference it synchronises once the fields are on the device. */
 LBMRV_API int lbmrv_init_equilibrium_host(lbmrv_t h, const float* rho_host, const float* u_host);
 
-/* Advance n >= 0 time steps. Each step is one fused kernel: pull transport of the
- * previous post-relaxation state (relation (transport)), then the relaxation in the
- * frame moving at u~ (relation (relaxationu)) done as
+/* Advance n >= 0 time steps. Each step is pull transport of the previous post-relaxation
+ * state (relation (transport)), then the relaxation in the frame moving at u~ (relation
+ * (relaxationu)) done as
  *   m0 = M(0) f, d = m0 - m_eq(0), f* = f - M(0)^{-1} T(-u~) S T(u~) d
- * with T from Appendix A. Step k relaxes at time index t = k. */
+ * with T from Appendix A. Step k relaxes at time index t = k. One fused kernel does one
+ * step, or, with the automatic kernel variant, several steps of one call (D2Q9); the states
+ * are the same bit for bit, and n steps leave the state in the buffer that n calls of one
+ * step would leave it in. */
 LBMRV_API int lbmrv_step(lbmrv_t h, int64_t n);
 
 /* Density and velocity u = q/rho (relation (rhoq)) of the current state.

@@ -21,11 +21,13 @@ namespace {
 // BASIS 0: the orthogonal moments of relation (mom); 1: Geier's basis (relax_node_geier).
 // For BASIS 0 the relaxation takes u~ = q / rho itself (UM_FLUID) and ignores u~ for
 // UM_ZERO, so only the prescribed modes evaluate relative_velocity first.
-template <int BASIS, int UM, int RCP>
+template <typename T, int BASIS, int UM, int RCP>
 __device__ __forceinline__ void relax_basis(float g[9], float ux, float uy, const Rates& s,
                                             const StoreRef& ref) {
     if constexpr (BASIS == 0)
         relax_node<UM, RCP>(g, ux, uy, s, ref);
+    else if constexpr (sizeof(T) == 4)
+        relax_node_geier_r<UM, RCP_RN>(g, ux, uy, s, ref);
     else
         relax_node_geier(g, ux, uy, s, ref);
 }
@@ -117,7 +119,7 @@ __global__ void __launch_bounds__(256) k_step_scalar(const T* __restrict__ src,
         float ux = 0.0f, uy = 0.0f;
         if constexpr (needs_utilde<BASIS, UM>())
             relative_velocity<UM>(g, a.ref, x, y, r0 + x, a, ux, uy);
-        relax_basis<BASIS, UM, scalar_rcp<T>()>(g, ux, uy, a.s, a.ref);
+        relax_basis<T, BASIS, UM, scalar_rcp<T>()>(g, ux, uy, a.s, a.ref);
 #pragma unroll
         for (int j = 0; j < 9; ++j) dst[j * n + r0 + x] = from_f<T>(g[j]);
     }
@@ -223,7 +225,7 @@ __global__ void __launch_bounds__(128, (step_vec_min_blocks<T, BASIS, NV, UM, SU
                     } else if constexpr (needs_utilde<BASIS, UM>()) {
                         relative_velocity<UM>(h, a.ref, p.x0 + k, y, r0 + p.x0 + k, a, ux, uy);
                     }
-                    relax_basis<BASIS, UM, scalar_rcp<T>()>(h, ux, uy, a.s, a.ref);
+                    relax_basis<T, BASIS, UM, scalar_rcp<T>()>(h, ux, uy, a.s, a.ref);
 #pragma unroll
                     for (int j = 0; j < 9; ++j) g[j][k] = h[j];
                 }

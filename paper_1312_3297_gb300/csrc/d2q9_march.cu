@@ -1,0 +1,380 @@
+// D2Q9: three time steps per pass over memory (temporal blocking in the row direction).
+//
+// One step reads and writes every population once and runs at the copy bandwidth, so a run of
+// n steps costs n times the state's traffic although only the first and the last state are
+// wanted. k_march3 carries each row of a strip through three relaxations before it is stored:
+// a warp marches up a strip of 32 packs (4 nodes each); when level 1 has relaxed row r, level
+// 2 can relax row r - 1 and level 3 row r - 2, from the populations the level below left one
+// and two rows ago (a delay line in shared memory) and just now (registers). The arithmetic of
+// a node is that of the one-step kernels, in storage precision between the levels, so the
+// states are theirs bit for bit.
+//
+// What bounds it: the FP32 pipe, 68 % busy at 4096^2 (ncu; 55 % of issue slots, DRAM at 5 TB/s).
+// A packed multiply-add of three distinct register pairs takes it 3 cycles instead of 2 (24.7
+// against 36.6 T lane operations/s measured), and 1.06 - 1.16 relaxations are done per stored
+// one (lanes 0 and 31, the rows below a segment). Scalar multiply-adds in place of the packed
+// ones, three warps per scheduler instead of four, and two or four levels were slower (FP32
+// 4096^2: 150 k MLUPS with two levels, 203 k with four). Steps per pass are odd so that every
+// state lands in the buffer in which as many single steps would leave it.
+// Measured, MLUPS, u~ = q/rho, one step per launch -> here: FP32 3072^2 95 k -> 204 k, 2048^2
+// 91 k -> 177 k; FP16 8192^2 184 k -> 215 k, 2048^2 164 k -> 173 k; BF16 8192^2 185 k -> 227 k.
+#include <cuda_runtime.h>
+
+#include <atomic>
+
+#include "async_copy.cuh"
+#include "d2q9.cuh"
+#include "launch.h"
+#include "occupancy.cuh"
+#include "pdl.cuh"
+#include "pull.cuh"
+
+namespace lbmrv {
+namespace {
+
+// Warps per block, on neighbouring strips of the same rows (measured: FP32 4096^2 204 k MLUPS
+// with two against 201 k with one; 16-bit 8192^2 227 k with one against 221 k with two).
+template <typename T>
+constexpr int kWarps = sizeof(T) == 4 ? 2 : 1;
+template <typename T>
+constexpr int kThreads = 32 * kWarps<T>;
+constexpr int kLevels = kMarchSteps;
+constexpr int kNV = 4;  // nodes per pack
+// Packs of a strip that are stored: each level loses one node at both ends of a strip, whose
+// neighbours belong to the next strips, so lanes 0 and 31 are recomputed there (kLevels <= kNV
+// + 1 keeps the loss within those lanes).
+constexpr int kUse = 30;
+constexpr int64_t kMarchMinBytes = 128 << 20;  // about the L2 (129 MB)
+
+// A pack in storage form: NV consecutive nodes in W 32-bit words.
+template <typename T>
+constexpr int kW = kNV * (int)sizeof(T) / 4;
+
+template <typename T>
+__device__ __forceinline__ F2 get_pair(const uint32_t* w, int k) {
+    if constexpr (sizeof(T) == 4) {
+        return pack2(__uint_as_float(w[2 * k]), __uint_as_float(w[2 * k + 1]));
+    } else {
+        const float2 f = Cvt16<T>::unpack(w[k]);
+        return pack2(f.x, f.y);
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void put_pair(uint32_t* w, int k, F2 v) {
+    float a, b;
+    unpack2(v, a, b);
+    if constexpr (sizeof(T) == 4) {
+        w[2 * k] = __float_as_uint(a);
+        w[2 * k + 1] = __float_as_uint(b);
+    } else {
+        w[k] = Cvt16<T>::pack(a, b);
+    }
+}
+
+// (prev, v0, ..., v_{NV-2}), prev from the left lane.
+template <typename T>
+__device__ __forceinline__ void from_left(uint32_t v[kW<T>]) {
+    constexpr int W = kW<T>;
+    const uint32_t p = __shfl_up_sync(kFullMask, v[W - 1], 1);
+#pragma unroll
+    for (int i = W - 1; i >= 0; --i) {
+        const uint32_t l = i ? v[i - 1] : p;
+        v[i] = sizeof(T) == 4 ? l : __byte_perm(l, v[i], 0x5432);
+    }
+}
+// (v1, ..., v_{NV-1}, next), next from the right lane.
+template <typename T>
+__device__ __forceinline__ void from_right(uint32_t v[kW<T>]) {
+    constexpr int W = kW<T>;
+    const uint32_t p = __shfl_down_sync(kFullMask, v[0], 1);
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        const uint32_t r = i < W - 1 ? v[i + 1] : p;
+        v[i] = sizeof(T) == 4 ? r : __byte_perm(v[i], r, 0x5432);
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void shift_x(uint32_t g[9][kW<T>]) {
+    from_left<T>(g[1]);
+    from_right<T>(g[3]);
+    from_left<T>(g[5]);
+    from_right<T>(g[6]);
+    from_right<T>(g[7]);
+    from_left<T>(g[8]);
+}
+
+template <int W>
+struct alignas(4 * W) Words {
+    uint32_t w[W];
+};
+template <int W>
+__device__ __forceinline__ void ldw(const void* p, uint32_t w[W]) {
+    const Words<W> v = *reinterpret_cast<const Words<W>*>(p);
+#pragma unroll
+    for (int i = 0; i < W; ++i) w[i] = v.w[i];
+}
+template <int W>
+__device__ __forceinline__ void stw(void* p, const uint32_t w[W]) {
+    Words<W> v;
+#pragma unroll
+    for (int i = 0; i < W; ++i) v.w[i] = w[i];
+    *reinterpret_cast<Words<W>*>(p) = v;
+}
+
+// The relaxation of one pack held in storage form, two nodes per packed FP32 instruction.
+// amp: the prescribed field's factor; cx, cy: its base field on the pack (analytic: cx[0] for
+// the whole row).
+template <typename T, int UM, int BASIS, int RCP>
+__device__ __forceinline__ void relax_pack(uint32_t g[9][kW<T>], float amp, const float* cx,
+                                           const float* cy, const StepArgs& a) {
+#pragma unroll
+    for (int k = 0; k < kNV / 2; ++k) {
+        F2 h[9];
+#pragma unroll
+        for (int j = 0; j < 9; ++j) h[j] = get_pair<T>(g[j], k);
+        F2 ux(0.0f), uy(0.0f);
+        if constexpr (UM == UM_ANALYTIC) {
+            ux = F2(amp * cx[0]);
+            uy = F2(amp) * pack2(cy[2 * k], cy[2 * k + 1]);
+        } else if constexpr (UM == UM_FIELD) {
+            ux = F2(amp) * pack2(cx[2 * k], cx[2 * k + 1]);
+            uy = F2(amp) * pack2(cy[2 * k], cy[2 * k + 1]);
+        }
+        if constexpr (BASIS == 0)
+            relax_node<UM, RCP>(h, ux, uy, a.s, a.ref);
+        else
+            relax_node_geier_r<UM, RCP>(h, ux, uy, a.s, a.ref);
+#pragma unroll
+        for (int j = 0; j < 9; ++j) put_pair<T>(g[j], k, h[j]);
+    }
+}
+
+// Shared memory, private to each thread: the next row's nine packs, and nine packs of delay
+// line per level but the last; a stored field adds its next row's two packs.
+template <typename T>
+constexpr int kSlot = kThreads<T> * 4 * kW<T>;
+template <typename T, int UM>
+constexpr int kSmem = kSlot<T> * 9 * kLevels + (UM == UM_FIELD ? 2 * kThreads<T> * 16 : 0);
+// 16 warps per SM (128 registers, no spills); 12 with a stored field, whose rows of the three
+// levels stay in registers.
+template <typename T, int UM>
+constexpr int kBlocks = (UM == UM_FIELD ? 12 : 16) / kWarps<T>;
+
+template <typename T, int UM, int BASIS, int RCP>
+__global__ void __launch_bounds__(kThreads<T>, (kBlocks<T, UM>))
+    k_march3(const T* __restrict__ src, T* __restrict__ dst, StepArgs a, MarchAmps amps,
+             int groups, int segs) {
+    extern __shared__ __align__(16) char smem[];
+    pdl_wait_prior();
+    pdl_allow_next();
+    constexpr int W = kW<T>, SB = kSlot<T>;
+    const int nx = a.nx, ny = a.ny;
+    const int64_t n = (int64_t)nx * ny;
+    const int lane = threadIdx.x & 31;
+    const int grp = blockIdx.x % groups, seg = blockIdx.x / groups;
+    const int packs = nx / kNV;
+    const int pk = (grp * kWarps<T> + (threadIdx.x >> 5)) * kUse + lane - 1;
+    const bool act = lane >= 1 && lane <= kUse && pk < packs;
+    int pw = pk % packs;  // lanes past the row's ends take its periodic continuation
+    if (pw < 0) pw += packs;
+    const int x0 = pw * kNV;
+    const int y0 = (int)((int64_t)seg * ny / segs), y1 = (int)((int64_t)(seg + 1) * ny / segs);
+    char* const mine = smem + threadIdx.x * (4 * W);
+    char* const field = smem + 9 * kLevels * SB + threadIdx.x * 16;
+    const T* const s0 = src + x0;
+    auto load_row = [&](int64_t om, int64_t o0, int64_t op) {
+        const int64_t row[3] = {om, o0, op};
+        constexpr int dy[9] = {1, 1, 0, 1, 2, 0, 0, 2, 2};  // row[1 - c_y]
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            if constexpr (W == 4)
+                cp_async16(mine + j * SB, s0 + j * n + row[dy[j]]);
+            else
+                cp_async8(mine + j * SB, s0 + j * n + row[dy[j]]);
+        }
+        if constexpr (UM == UM_FIELD) {
+            cp_async16(field, a.ut0 + o0 + x0);
+            cp_async16(field + kThreads<T> * 16, a.ut0 + n + o0 + x0);
+        }
+        cp_async_commit();
+    };
+    auto up = [&](int y) { return y == ny - 1 ? 0 : y + 1; };
+    // u~0 on the rows of the three levels: the analytic field's cos 2 pi y/ny per row and sin
+    // 2 pi x/nx per column, or a stored field's packs
+    float bx[kLevels][UM == UM_FIELD ? kNV : 1], by[UM == UM_FIELD ? kLevels : 1][kNV];
+    if constexpr (UM == UM_ANALYTIC) {
+#pragma unroll
+        for (int k = 0; k < kNV; ++k) by[0][k] = __ldg(a.sin_x + x0 + k);
+    }
+    // rows r - 1, r, r + 1 of the row that level 1 relaxes next
+    int r = y0 - (kLevels - 1);
+    while (r < 0) r += ny;
+    int rm = r == 0 ? ny - 1 : r - 1, rp = up(r);
+    int out = y0;
+    const int rows = y1 - y0 + 2 * (kLevels - 1);
+    load_row((int64_t)rm * nx, (int64_t)r * nx, (int64_t)rp * nx);
+    for (int i = 0; i < rows; ++i) {
+        const int rq = up(rp);
+        cp_async_wait_all_but<0>();
+        uint32_t g[9][W];
+#pragma unroll
+        for (int j = 0; j < 9; ++j) ldw<W>(mine + j * SB, g[j]);
+        if constexpr (UM == UM_ANALYTIC) {
+#pragma unroll
+            for (int l = kLevels - 1; l > 0; --l) bx[l][0] = bx[l - 1][0];
+            bx[0][0] = cospif(a.two_over_ny * (float)(r + a.y_off));
+        } else if constexpr (UM == UM_FIELD) {
+#pragma unroll
+            for (int k = 0; k < kNV; ++k) {
+#pragma unroll
+                for (int l = kLevels - 1; l > 0; --l) {
+                    bx[l][k] = bx[l - 1][k];
+                    by[l][k] = by[l - 1][k];
+                }
+            }
+            ldw<kNV>(field, reinterpret_cast<uint32_t*>(bx[0]));
+            ldw<kNV>(field + kThreads<T> * 16, reinterpret_cast<uint32_t*>(by[0]));
+        }
+        shift_x<T>(g);
+        relax_pack<T, UM, BASIS, RCP>(g, amps.v[0], bx[0], by[0], a);
+        // the slots have been read: fetch the next row behind levels 2 and 3
+        if (i + 1 < rows) load_row((int64_t)r * nx, (int64_t)rp * nx, (int64_t)rq * nx);
+#pragma unroll
+        for (int l = 1; l < kLevels; ++l) {
+            if (i < 2 * (l - 1)) continue;
+            // the row below: {0,1,3} as level l left them one row ago, {2,5,6} two rows ago
+            // (a ring of two), {4,7,8} now
+            shift_x<T>(g);
+            char* const d = mine + 9 * l * SB;
+            char* const e = d + (3 + 3 * (i & 1)) * SB;
+            constexpr int c0[3] = {0, 1, 3}, cp[3] = {2, 5, 6};
+            uint32_t q[6][W];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                ldw<W>(d + c * SB, q[c]);
+                ldw<W>(e + c * SB, q[3 + c]);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                stw<W>(d + c * SB, g[c0[c]]);
+                stw<W>(e + c * SB, g[cp[c]]);
+            }
+            if (i < 2 * l) continue;  // the delay line is not yet full
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    g[c0[c]][w] = q[c][w];
+                    g[cp[c]][w] = q[3 + c][w];
+                }
+            }
+            relax_pack<T, UM, BASIS, RCP>(g, amps.v[l], bx[l], by[UM == UM_FIELD ? l : 0], a);
+        }
+        if (i >= 2 * (kLevels - 1)) {
+            if (act) {
+                T* const d = dst + (int64_t)out * nx + x0;
+#pragma unroll
+                for (int j = 0; j < 9; ++j) stw<W>(d + j * n, g[j]);
+            }
+            ++out;
+        }
+        rm = r;
+        r = rp;
+        rp = rq;
+    }
+}
+
+template <typename T, int UM, int BASIS, int RCP>
+cudaError_t launch_t(const void* src, void* dst, const StepArgs& a, const MarchAmps& amps,
+                     cudaStream_t st) {
+    const int packs = a.nx / kNV;
+    const int groups = (packs + kWarps<T> * kUse - 1) / (kWarps<T> * kUse);
+    auto kernel = k_march3<T, UM, BASIS, RCP>;
+    static std::atomic<int> resident[kMaxDevicesOcc];
+    int full = 0;
+    cudaError_t e = resident_blocks(kernel, resident, kThreads<T>, kSmem<T, UM>, 32, &full);
+    if (e != cudaSuccess) return e;
+    // One segment of rows per resident block and strip group. Segments under 8 rows repeat too
+    // many relaxations (2 (kLevels - 1) rows each): half as many then (FP32 1536 x 1000 145 k
+    // MLUPS against 138 k). Long 16-bit segments are halved, so that blocks that end early leave
+    // work to take (8192^2 227 k against 224 k; no gain in FP32).
+    int64_t segs = full / groups;
+    if (segs * 8 > a.ny) segs = full / 2 / groups;
+    if (sizeof(T) == 2 && segs * 64 < a.ny) segs = 2 * segs;
+    if (segs > a.ny) segs = a.ny;
+    if (segs < 1) segs = 1;
+    e = launch_pdl_smem(kernel, dim3((unsigned)(groups * segs)), dim3(kThreads<T>), kSmem<T, UM>, st,
+                        static_cast<const T*>(src), static_cast<T*>(dst), a, amps, groups,
+                        (int)segs);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// 1/rho in the form that the one-step kernel of the same rows uses (d2q9_kernels.cu), so that
+// both give the same bits: FP32 the approximation (Geier's basis: correctly rounded); 16-bit
+// rows of 8-node packs, and Geier's 4-node packs, the paired form; other 16-bit rows the
+// correctly rounded one.
+template <typename T, int BASIS, int UM>
+cudaError_t launch_rcp(const void* s, void* d, const StepArgs& a, const MarchAmps& amps,
+                       cudaStream_t st) {
+    if constexpr (sizeof(T) == 4) {
+        return launch_t<T, UM, BASIS, BASIS == 0 ? RCP_APPROX : RCP_RN>(s, d, a, amps, st);
+    } else if constexpr (UM == UM_ZERO) {
+        return launch_t<T, UM, BASIS, RCP_RN>(s, d, a, amps, st);
+    } else {
+        if constexpr (BASIS == 0) {
+            if (a.nx % 8 != 0) return launch_t<T, UM, BASIS, RCP_RN>(s, d, a, amps, st);
+        }
+        return launch_t<T, UM, BASIS, RCP_DIV>(s, d, a, amps, st);
+    }
+}
+
+template <typename T, int BASIS>
+cudaError_t launch_um(int um, const void* s, void* d, const StepArgs& a, const MarchAmps& amps,
+                      cudaStream_t st) {
+    switch (um) {
+        case UM_ZERO: return launch_rcp<T, BASIS, UM_ZERO>(s, d, a, amps, st);
+        case UM_FLUID: return launch_rcp<T, BASIS, UM_FLUID>(s, d, a, amps, st);
+        case UM_ANALYTIC: return launch_rcp<T, BASIS, UM_ANALYTIC>(s, d, a, amps, st);
+        case UM_FIELD: return launch_rcp<T, BASIS, UM_FIELD>(s, d, a, amps, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+template <typename T>
+cudaError_t launch_basis(int um, const void* s, void* d, const StepArgs& a,
+                         const MarchAmps& amps, cudaStream_t st, int basis) {
+    return basis == 0 ? launch_um<T, 0>(um, s, d, a, amps, st)
+                      : launch_um<T, 1>(um, s, d, a, amps, st);
+}
+
+}  // namespace
+
+bool march_usable(int storage, int um, int basis, int nx, int ny, const void* a, const void* b,
+                  const float* ut0) {
+    const int bytes = storage == kStoreF32 ? 16 : 8;
+    if (nx % kNV != 0 || reinterpret_cast<uintptr_t>(a) % bytes != 0 ||
+        reinterpret_cast<uintptr_t>(b) % bytes != 0)
+        return false;
+    if (um == UM_FIELD && (reinterpret_cast<uintptr_t>(ut0) % 16 != 0 ||
+                           (storage != kStoreF32 && basis == 1 && nx % 8 != 0)))
+        return false;
+    // While both states stay in L2 a single step is not bound by DRAM and the repeated
+    // relaxations cost more than the traffic saved: FP32 1024^2 (75 MB of states) 124 k MLUPS
+    // either way, 1448^2 (151 MB) 88 k -> 141 k; 16-bit 1024 x 2048 (75 MB) 198 k against 169 k
+    // here, 2048^2 (151 MB) 165 k -> 182 k.
+    return 2 * 9 * (int64_t)nx * ny * (storage == kStoreF32 ? 4 : 2) > kMarchMinBytes;
+}
+
+cudaError_t launch_march(int storage, int um, const void* src, void* dst, const StepArgs& a,
+                         const MarchAmps& amps, cudaStream_t st, int basis) {
+    switch (storage) {
+        case kStoreF32: return launch_basis<float>(um, src, dst, a, amps, st, basis);
+        case kStoreF16: return launch_basis<__half>(um, src, dst, a, amps, st, basis);
+        case kStoreBF16: return launch_basis<__nv_bfloat16>(um, src, dst, a, amps, st, basis);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace lbmrv

@@ -105,6 +105,11 @@ inline double time_factor(const lbmrv_s* h, int64_t t) {
     return h->period > 0.0 ? std::cos(2.0 * M_PI * (double)t / h->period) : 1.0;
 }
 
+// The prescribed field's factor A cos(2 pi t / P) / lambda at time index t.
+inline float prescribed_amp(const lbmrv_s* h, int64_t t) {
+    return (float)(h->amp * time_factor(h, t) / h->lambda);
+}
+
 // Reference state of the stored deviations, lattice units (see StoreRef in d2q9.cuh).
 inline StoreRef store_ref(const lbmrv_s* h) {
     const double r = h->rho_ref;
@@ -167,7 +172,7 @@ inline StepArgs make_args(const lbmrv_s* h, int64_t t) {
     a.s = Rates{(float)h->s[3], (float)h->s[4], (float)h->s[5],
                 (float)h->s[6], (float)h->s[7], (float)h->s[8]};
     a.ref = store_ref(h);
-    a.amp_t = (float)(h->amp * time_factor(h, t) / h->lambda);
+    a.amp_t = prescribed_amp(h, t);
     a.two_over_nx = (float)(2.0 / (double)h->nx);
     // a slab evaluates the analytic field at the global row: y + y_off of slab_extent rows
     a.two_over_ny = (float)(2.0 / (double)(h->slab ? h->slab_extent : h->ny));
@@ -188,7 +193,7 @@ inline StepArgs3 make_args3(const lbmrv_s* h, int64_t t) {
                  (float)s[9],  (float)s[10], (float)s[11], (float)s[12], (float)s[13],
                  (float)s[14], (float)s[15], (float)s[16], (float)s[17], (float)s[18]};
     a.ref = store_ref3(h);
-    a.amp_t = (float)(h->amp * time_factor(h, t) / h->lambda);
+    a.amp_t = prescribed_amp(h, t);
     a.ut0 = h->ut0;
     return a;
 }

@@ -32,6 +32,18 @@ int step_vector_width(int storage, int nx);
 cudaError_t launch_step(int storage, int um, int nv, const void* src, void* dst,
                         const StepArgs& a, cudaStream_t st, int basis = 0);
 
+// kMarchSteps steps src -> dst in one pass over memory (d2q9_march.cu), the bits of that many
+// launch_step calls. a: the arguments of the first of them; amps: amp_t of each.
+// march_usable: whether the lattice suits it (u~0 the stored field, or null).
+constexpr int kMarchSteps = 3;
+struct MarchAmps {
+    float v[kMarchSteps];
+};
+bool march_usable(int storage, int um, int basis, int nx, int ny, const void* a, const void* b,
+                  const float* ut0);
+cudaError_t launch_march(int storage, int um, const void* src, void* dst, const StepArgs& a,
+                         const MarchAmps& amps, cudaStream_t st, int basis);
+
 // The same step (nv >= 2) with the FP64 conserved sums of dst fused in, written to out[4]
 // as launch_conserved does; partials: step_sum_scratch(nx, ny, nv) doubles of scratch.
 int64_t step_sum_blocks(int nx, int ny, int nv);
