@@ -212,9 +212,9 @@ LBMRV_API int lbmrv_init_equilibrium_host(lbmrv_t h, const float* rho_host, cons
  * (relaxationu)) done as
  *   m0 = M(0) f, d = m0 - m_eq(0), f* = f - M(0)^{-1} T(-u~) S T(u~) d
  * with T from Appendix A. Step k relaxes at time index t = k. One fused kernel does one
- * step, or, with the automatic kernel variant, several steps of one call (D2Q9); the states
- * are the same bit for bit, and n steps leave the state in the buffer that n calls of one
- * step would leave it in. */
+ * step, or, with the automatic kernel variant, several steps of one call (D2Q9, 3 or more
+ * steps, chosen by lattice size, storage and row length); the states are the same bit for
+ * bit, and n steps leave the state in the buffer that n calls of one step would leave it in. */
 LBMRV_API int lbmrv_step(lbmrv_t h, int64_t n);
 
 /* Density and velocity u = q/rho (relation (rhoq)) of the current state.

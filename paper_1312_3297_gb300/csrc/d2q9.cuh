@@ -152,7 +152,12 @@ __device__ __forceinline__ F1 recip(F1 x) {
 // T(u~) acts: identity on (e, p_xx, p_xy) plus C3 (rows q_x, q_y), D3 and D4 (row eps)
 // of Appendix A. Then f* = f - M(0)^{-1} T(-u~) S T(u~) d, where M(0)^{-1} =
 // M(0)^T diag(1/|row|^2) with |row|^2 = 36, 4, 4, 12, 12, 36 on the six moments.
-template <int UM, int RCP = RCP_RN, typename R>
+//
+// ux^2 - uy^2 is the one place where two products could be fused with the subtraction; the
+// compiler fuses the first, but the second where the first is shared by a row of nodes (the
+// packs of the analytic field). ROW spells out that second form, for kernels that must give
+// the same bits with another loop order.
+template <int UM, int RCP = RCP_RN, bool ROW = false, typename R>
 LBMRV_HD void relax_node(R g[9], R& ux, R& uy, const Rates& s, const StoreRef& ref) {
     // Sums and differences of opposite populations.
     const R a1 = g[1] + g[3], b1 = g[1] - g[3], a2 = g[2] + g[4], b2 = g[2] - g[4];
@@ -194,7 +199,8 @@ LBMRV_HD void relax_node(R g[9], R& ux, R& uy, const Rates& s, const StoreRef& r
         const R ux2 = ux + ux, uy2 = uy + uy, ux3 = ux2 + ux, uy3 = uy2 + uy;
         const R ux6 = ux3 + ux3, uy6 = uy3 + uy3;
         const R d3e = fma_(ux6, ux, uy6 * uy);       // 6 |u|^2
-        const R d3xx = ux3 * ux3 - uy3 * uy3;        // 9 (ux^2 - uy^2)
+        const R d3xx = ROW ? fma_(R(0.0f) - uy3, uy3, ux3 * ux3)
+                           : ux3 * ux3 - uy3 * uy3;  // 9 (ux^2 - uy^2)
         const R d3xy = ux6 * uy6;                    // 36 ux uy
         // Forward shift T(u~) d, then the diagonal relaxation S.
         const R t_qx = d_qx - fma_(ux2, d_e, fma_(ux3, d_pxx, uy6 * d_pxy));

@@ -1,0 +1,136 @@
+// The tile kernel's plan and its FP32 instances (d2q9_tile.cuh).
+#include "d2q9_tile.cuh"
+
+namespace lbmrv {
+
+namespace {
+
+// Times in microseconds measured on GB300, for the choice of a plan only (any plan gives the
+// same states).
+constexpr double kLaunch = 2.1;      // a pass: launch, first loads, last stores
+constexpr double kStepFloor = 0.46;  // a step of a block that fills no pipe
+constexpr double kItem = 0.0545;     // a warp's two rows of 32 nodes on a busy SM, per SM
+constexpr double kSerial = 2.0;      // loads and stores of a tile that nothing else overlaps
+
+bool fits_l2(double nodes, int node_bytes) { return 2.0 * node_bytes * nodes < 128e6; }
+
+// A single-step launch: the launch and the time per million nodes at its pack width, with the
+// states in L2 or in DRAM.
+double single_step_us(int storage, int nv, double nodes, int node_bytes) {
+    const bool l2 = fits_l2(nodes, node_bytes);
+    double per_m;
+    if (storage == kStoreF32)
+        per_m = nv == 4 ? (l2 ? 6.4 : 10.5) : nv == 2 ? (l2 ? 8.2 : 10.9) : (l2 ? 7.7 : 11.2);
+    else
+        per_m = nv == 8 ? (l2 ? 4.4 : 5.8) : nv == 4 ? 6.7 : nv == 2 ? 7.7 : 9.5;
+    return 1.9 + per_m * 1e-6 * nodes;
+}
+
+int sm_count() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        return 152;
+    return sms;
+}
+
+}  // namespace
+
+// The plan with the least modelled time for n steps: steps per pass, array size and warps per
+// block. Small lattices take many steps per pass (64^2: 10, over 32 x 22 arrays), since a launch
+// costs as much as four steps; larger ones the array whose tiles just fill the SMs (512^2: 4 over
+// 64 x 38). Aligned rows of larger L2-resident lattices stay with single steps, which the
+// repeated relaxations of the halos would not beat (FP32 1024^2 8.5 us a step against 9.4,
+// 16-bit 768^2 5.0 against 5.6); there is no such limit for rows without vector packs.
+// Measured, single steps -> here, us a step (u~ = q/rho): FP32 64^2 2.05 -> 0.82, 256^2 2.3 ->
+// 1.22, 512^2 3.9 -> 2.73, 1023^2 10.1 -> 8.3, 4097 x 1999 94 -> 60; FP16 64^2 2.1 -> 0.87,
+// 512^2 3.0 -> 2.9, 513 x 511 4.5 -> 2.9, 4097 x 1999 82 -> 60.
+TilePlan tile_plan(int storage, int um, int nv, int nx, int ny, int64_t n) {
+    TilePlan best;
+    const int elem = storage == kStoreF32 ? 4 : 2, sms = sm_count();
+    const double nodes = (double)nx * ny;
+    const bool in_l2 = fits_l2(nodes, 9 * elem);
+    const double per_sm = kItem / sms;
+    // only where clearly less than single steps
+    double least = 0.93 * n * single_step_us(storage, nv, nodes, 9 * elem);
+    // likely lengths first: a good plan early drops most of the others unevaluated
+    constexpr int lengths[] = {5, 10, 4, 3, 8, 6, 12, 2};
+    constexpr int heights[] = {12, 16, 20, 22, 24, 26, 28, 32, 36, 38, 40, 44, 46, 48, 56, 62};
+    for (int want : lengths) {
+        // an odd number of passes for an odd number of steps, an even one for an even number:
+        // the state ends in the buffer in which single steps would leave it
+        int64_t m = (n + want - 1) / want;
+        m += (m ^ n) & 1;
+        const int s = (int)((n + m - 1) / m);
+        if (s < 2) continue;
+        for (int rx = 32; rx <= 64; rx += 32) {
+            const int tx = rx - 2 * (s - 1);
+            if (tx < 4) continue;
+            const int tiles_x = (nx + tx - 1) / tx;
+            for (int ry : heights) {
+                const int ty = ry - 2 * (s - 1);
+                if (ty < 4) continue;
+                const int bytes = (int)tile_bytes(rx, ry, elem, um);
+                if (bytes > kTileMaxSmem || ty > ny + 8) break;
+                const int tiles = tiles_x * ((ny + ty - 1) / ty);
+                // the pipes' share of a pass, were its tiles spread evenly: usually enough to
+                // drop a candidate
+                const double even = per_sm * s * (rx / 32) * ((ry + ty) / 4) * tiles;
+                const double steps_alone = kStepFloor * s;
+                if (m * (kLaunch + (even > steps_alone ? even : steps_alone)) >= least) continue;
+                const int items = rx / 32 * (ry / 2);
+                const int rounds = (items + kTileWarps - 1) / kTileWarps;
+                const int whole = (items + rounds - 1) / rounds;
+                // one block per SM with a warp for every item, or several with half as many
+                for (int half = 1; half <= 2; ++half) {
+                    int warps = (whole + half - 1) / half;
+                    warps = (warps + rx / 32 - 1) / (rx / 32) * (rx / 32);
+                    int fit = (227 * 1024) / (bytes + 1024);
+                    if (fit > kTileWarps / warps) fit = kTileWarps / warps;
+                    if (fit < 1) continue;
+                    // the first step's loads: latency that few later steps leave exposed
+                    const double first = (s == 2 ? (in_l2 ? 1.5 : 2.0) : s == 3 ? 1.2 : 1.0) +
+                                         (um == UM_FIELD ? 0.8 : 0.0);
+                    // `resident` tiles at a time on an SM
+                    auto wave = [&](int resident) {
+                        const double busy = (double)resident * warps;
+                        const double item =
+                            kItem * (busy < 20.0 ? 1.0 + 0.03 * (20.0 - busy) : 1.0);
+                        double us = 0.0;
+                        for (int k = 0; k < s; ++k) {
+                            const int pairs = rx / 32 * ((ry - k - 1) / 2 - k / 2 + 1);
+                            const double pipes = (k ? 1.0 : first) * item * pairs * resident;
+                            const double alone =
+                                pairs <= warps ? kStepFloor
+                                               : kStepFloor * ((pairs + warps - 1) / warps);
+                            us += pipes > alone ? pipes : alone;
+                        }
+                        return us;
+                    };
+                    const int full = tiles / (sms * fit), rest = tiles - full * sms * fit;
+                    double us = full * wave(fit) + (rest ? wave((rest + sms - 1) / sms) : 0.0);
+                    if (fit == 1 && tiles > sms) us += kSerial * (tiles - sms) / sms;
+                    const double total = m * (kLaunch + us);
+                    if (total < least) {
+                        least = total;
+                        best.steps = s;
+                        best.rx = rx;
+                        best.ry = ry;
+                        best.warps = warps;
+                        best.launches = m;
+                    }
+                }
+            }
+        }
+    }
+    return best;
+}
+
+cudaError_t launch_tile(int storage, int um, int basis, int nv, const void* src, void* dst,
+                        const StepArgs& a, const TileAmps& amps, const TilePlan& p,
+                        cudaStream_t st) {
+    if (storage == kStoreF32) return tile_basis<float>(um, basis, nv, src, dst, a, amps, p, st);
+    return launch_tile16(storage, um, basis, nv, src, dst, a, amps, p, st);
+}
+
+}  // namespace lbmrv

@@ -38,6 +38,9 @@ struct lbmrv_s {
     int64_t t = 0;
     const float* ut0 = nullptr;
     double amp = 0.0, period = 0.0;
+    int64_t tile_n = 0;   // the step count and mode that `tile` was planned for
+    int tile_um = -1;
+    lbmrv::TilePlan tile;
     double* red = nullptr;   // reduction scratch: 8 * red_blocks partials + 8 results
     int red_blocks = 0;
     double* fused = nullptr;  // partials of the step with fused sums, + 4 results (lazy)

@@ -44,6 +44,32 @@ bool march_usable(int storage, int um, int basis, int nx, int ny, const void* a,
 cudaError_t launch_march(int storage, int um, const void* src, void* dst, const StepArgs& a,
                          const MarchAmps& amps, cudaStream_t st, int basis);
 
+// p.steps steps src -> dst in one launch on shared-memory tiles (d2q9_tile.cuh): arrays of p.rx
+// x p.ry nodes, blocks of p.warps warps. The bits of that many launch_step calls at pack width nv.
+constexpr int kTileMaxSteps = 12;
+constexpr int kTileMinSteps = 5;  // of a call: fewer are not worth planning (about 10 us, once)
+constexpr int kTileMaxSmem = 224 * 1024;
+constexpr int kTileWarps = 24;  // most per block and per SM
+struct TileAmps {
+    float v[kTileMaxSteps];  // amp_t of each step
+};
+struct TilePlan {
+    int steps = 1;  // 1: single-step launches are faster
+    int rx = 0, ry = 0, warps = 0;
+    int64_t launches = 0;  // for the n steps planned: `launches` passes of at most `steps`
+};
+inline int64_t tile_bytes(int rx, int ry, int elem, int um) {
+    return 9LL * rx * (ry + 3) * elem +
+           (um == UM_FIELD ? 8LL * rx * (ry + 1) : um == UM_ANALYTIC ? 4LL * (ry + 1) : 0);
+}
+TilePlan tile_plan(int storage, int um, int nv, int nx, int ny, int64_t n);
+cudaError_t launch_tile(int storage, int um, int basis, int nv, const void* src, void* dst,
+                        const StepArgs& a, const TileAmps& amps, const TilePlan& p,
+                        cudaStream_t st);
+cudaError_t launch_tile16(int storage, int um, int basis, int nv, const void* src, void* dst,
+                          const StepArgs& a, const TileAmps& amps, const TilePlan& p,
+                          cudaStream_t st);
+
 // The same step (nv >= 2) with the FP64 conserved sums of dst fused in, written to out[4]
 // as launch_conserved does; partials: step_sum_scratch(nx, ny, nv) doubles of scratch.
 int64_t step_sum_blocks(int nx, int ny, int nv);

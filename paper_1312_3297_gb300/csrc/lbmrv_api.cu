@@ -382,6 +382,29 @@ int lbmrv_step(lbmrv_t h, int64_t n) {
             h->t += kMarchSteps;
         }
     }
+    // passes over shared-memory tiles, where they are faster than single steps; of equal
+    // lengths to within one
+    if (k == 0 && n >= kTileMinSteps && h->dim == 2 && h->width == 0 && !h->slab) {
+        const int um = kernel_mode(h);
+        if (h->tile_n != n || h->tile_um != um) {
+            h->tile = tile_plan(h->storage, um, nv, (int)h->nx, (int)h->ny, n);
+            h->tile_n = n;
+            h->tile_um = um;
+        }
+        TilePlan p = h->tile;
+        for (int64_t m = p.launches; m > 0; --m) {
+            p.steps = (int)((n - k + m - 1) / m);
+            TileAmps amps;
+            for (int l = 0; l < p.steps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);
+            cudaError_t e = launch_tile(h->storage, um, h->basis, nv, h->f[h->cur],
+                                        h->f[1 - h->cur], make_args(h, h->t + 1), amps, p,
+                                        h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step");
+            h->cur = 1 - h->cur;
+            h->t += p.steps;
+            k += p.steps;
+        }
+    }
     for (; k < n; ++k) {
         cudaError_t e = launch_handle_step(h, nv, h->f[h->cur], h->f[1 - h->cur], h->t + 1);
         if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step");
