@@ -200,6 +200,12 @@ LBMRV_API int lbmrv_set_utilde(lbmrv_t h, const float* ut0_dev, double amplitude
  * fields (the state is then left unchanged); LBMRV_E_CUDA. */
 LBMRV_API int lbmrv_init_equilibrium(lbmrv_t h, const float* rho_dev, const float* u_dev);
 
+/* Same with the velocity components in separate buffers: ux_dev, uy_dev and, for D3Q19, uz_dev
+ * (ignored otherwise), device FP32 [n] each. */
+LBMRV_API int lbmrv_init_equilibrium_fields(lbmrv_t h, const float* rho_dev,
+                                            const float* ux_dev, const float* uy_dev,
+                                            const float* uz_dev);
+
 /* Same from host buffers: copies them into the non-current state buffer on the
  * handle's stream (no allocation), then builds the equilibrium. Pinned host memory is
  * faster. With a fixed reference the call returns once the work is enqueued, and the host

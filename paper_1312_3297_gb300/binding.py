@@ -54,6 +54,7 @@ SIGNATURES = [
     ("lbmrv_set_kernel_width", _I, [_VP, _I]),
     ("lbmrv_set_utilde", _I, [_VP, _VP, _D, _D]),
     ("lbmrv_init_equilibrium", _I, [_VP, _VP, _VP]),
+    ("lbmrv_init_equilibrium_fields", _I, [_VP, _VP, _VP, _VP, _VP]),
     ("lbmrv_init_equilibrium_host", _I, [_VP, _VP, _VP]),
     ("lbmrv_step", _I, [_VP, _I64]),
     ("lbmrv_moments", _I, [_VP, _VP, _VP]),
@@ -198,6 +199,11 @@ def lbmrv_set_utilde(h, ut0, amplitude: float, period: float) -> None:
 
 def lbmrv_init_equilibrium(h, rho, u) -> None:
     _check(load().lbmrv_init_equilibrium(h, _addr(rho), _addr(u)), h)
+
+
+def lbmrv_init_equilibrium_fields(h, rho, ux, uy, uz=None) -> None:
+    _check(load().lbmrv_init_equilibrium_fields(h, _addr(rho), _addr(ux), _addr(uy), _addr(uz)),
+           h)
 
 
 def lbmrv_init_equilibrium_host(h, rho, u) -> None:

@@ -293,63 +293,74 @@ __device__ __forceinline__ float phi1(int c, float a) {
     return c == 0 ? (2.0f / 3.0f - a * a) : 0.5f * ((1.0f / 3.0f + a * a) + (float)c * a);
 }
 
-template <typename T>
-__global__ void k_init_eq_product(T* __restrict__ dst, const float* __restrict__ rho,
-                                  const float* __restrict__ u, int64_t n, StoreRef ref,
-                                  float inv_lambda) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+// NV consecutive nodes per thread (one vector access per plane), velocity components from
+// separate planes. BASIS 1: Geier's product equilibrium.
+template <typename T, int BASIS, int NV>
+__global__ void __launch_bounds__(256)
+    k_init_eq(T* __restrict__ dst, Fields fld, int64_t n, StoreRef ref, float inv_lambda) {
+    const int64_t packs = n / NV;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < packs;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const float r = rho ? rho[i] : 1.0f;
-        const float ux = u ? u[i] * inv_lambda : 0.0f;
-        const float uy = u ? u[n + i] * inv_lambda : 0.0f;
+        float r[NV], vx[NV], vy[NV], g[9][NV];
+        load_field<NV>(fld.rho, i, 1.0f, r);
+        load_field<NV>(fld.u[0], i, 0.0f, vx);
+        load_field<NV>(fld.u[1], i, 0.0f, vy);
 #pragma unroll
-        for (int j = 0; j < 9; ++j) {
-            const int cx = kCX[j], cy = kCY[j];
-            dst[j * n + i] = from_f<T>(r * phi1(cx, ux) * phi1(cy, uy) -
-                                       ref.rho * phi1(cx, ref.ux) * phi1(cy, ref.uy));
+        for (int k = 0; k < NV; ++k) {
+            const float ux = vx[k] * inv_lambda;
+            const float uy = vy[k] * inv_lambda;
+            if constexpr (BASIS == 1) {
+#pragma unroll
+                for (int j = 0; j < 9; ++j) {
+                    const int cx = kCX[j], cy = kCY[j];
+                    g[j][k] = r[k] * phi1(cx, ux) * phi1(cy, uy) -
+                              ref.rho * phi1(cx, ref.ux) * phi1(cy, ref.uy);
+                }
+            } else {
+                const float uu = ux * ux + uy * uy;
+                const float UU = ref.ux * ref.ux + ref.uy * ref.uy;
+                const float dr = r[k] - ref.rho;
+#pragma unroll
+                for (int j = 0; j < 9; ++j) {
+                    const float cu = (float)kCX[j] * ux + (float)kCY[j] * uy;
+                    const float cU = (float)kCX[j] * ref.ux + (float)kCY[j] * ref.uy;
+                    const float w = wgt(j);
+                    const float pu = 3.0f * cu + 4.5f * cu * cu - 1.5f * uu;
+                    const float pU = 3.0f * cU + 4.5f * cU * cU - 1.5f * UU;
+                    g[j][k] = w * dr + w * (r[k] * pu - ref.rho * pU);
+                }
+            }
         }
+#pragma unroll
+        for (int j = 0; j < 9; ++j) store_pack<T, NV>(dst + j * n + i * NV, g[j]);
     }
 }
 
-template <typename T>
-__global__ void k_init_eq(T* __restrict__ dst, const float* __restrict__ rho,
-                          const float* __restrict__ u, int64_t n, StoreRef ref,
-                          float inv_lambda) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+// Density and velocity (relation (rhoq)) of the stored state, NV consecutive nodes per thread.
+template <typename T, int NV>
+__global__ void __launch_bounds__(256)
+    k_moments(const T* __restrict__ src, float* __restrict__ rho, float* __restrict__ u,
+              int64_t n, StoreRef ref, float lambda) {
+    const int64_t packs = n / NV;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < packs;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const float r = rho ? rho[i] : 1.0f;
-        const float ux = u ? u[i] * inv_lambda : 0.0f;
-        const float uy = u ? u[n + i] * inv_lambda : 0.0f;
-        const float uu = ux * ux + uy * uy;
-        const float UU = ref.ux * ref.ux + ref.uy * ref.uy;
-        const float dr = r - ref.rho;
+        float g[9][NV], r[NV], ux[NV], uy[NV];
 #pragma unroll
-        for (int j = 0; j < 9; ++j) {
-            const float cu = (float)kCX[j] * ux + (float)kCY[j] * uy;
-            const float cU = (float)kCX[j] * ref.ux + (float)kCY[j] * ref.uy;
-            const float w = wgt(j);
-            const float pu = 3.0f * cu + 4.5f * cu * cu - 1.5f * uu;
-            const float pU = 3.0f * cU + 4.5f * cU * cU - 1.5f * UU;
-            dst[j * n + i] = from_f<T>(w * dr + w * (r * pu - ref.rho * pU));
+        for (int j = 0; j < 9; ++j) load_pack<T, NV>(src + j * n + i * NV, true, g[j]);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            float h[9];
+#pragma unroll
+            for (int j = 0; j < 9; ++j) h[j] = g[j][k];
+            const NodeMoments m = node_moments(h);
+            r[k] = ref.rho + m.drho;
+            ux[k] = lambda * (ref.jx + m.jx) / r[k];
+            uy[k] = lambda * (ref.jy + m.jy) / r[k];
         }
-    }
-}
-
-// Density and velocity (relation (rhoq)) of the stored state.
-template <typename T>
-__global__ void k_moments(const T* __restrict__ src, float* __restrict__ rho,
-                          float* __restrict__ u, int64_t n, StoreRef ref, float lambda) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        float g[9];
-#pragma unroll
-        for (int j = 0; j < 9; ++j) g[j] = to_f(src[j * n + i]);
-        const NodeMoments m = node_moments(g);
-        const float r = ref.rho + m.drho;
-        if (rho) rho[i] = r;
+        if (rho) store_pack<float, NV>(rho + i * NV, r);
         if (u) {
-            u[i] = lambda * (ref.jx + m.jx) / r;
-            u[n + i] = lambda * (ref.jy + m.jy) / r;
+            store_pack<float, NV>(u + i * NV, ux);
+            store_pack<float, NV>(u + n + i * NV, uy);
         }
     }
 }
@@ -421,21 +432,100 @@ __global__ void __launch_bounds__(kReduceThreads) k_conserved_final(const double
     }
 }
 
-// FP64 sums of rho, rho u_x, rho u_y and rho u_z (0 when dim = 2) over initial fields:
-// the total mass and momentum of the equilibrium state built from them (relation (rhoq)
-// summed over the lattice; sum_j v_j f_eq,j = rho u at every node). rho may be NULL
-// (rho = 1); u holds dim planes of n values.
+// Sum of FP32 terms kept in three FP32 parts whose sum is exact to about 2^-70 of it: the
+// rounding errors of the additions (and of the products) are carried along, by Knuth's two-sum
+// and Dekker's product with a fused multiply-add. Written with the single-operation
+// intrinsics, which the compiler does not contract.
+struct ExactSum {
+    float s = 0.0f, c = 0.0f, d = 0.0f;
+    static __device__ __forceinline__ float two_sum(float a, float b, float& e) {
+        const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+        e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+        return t;
+    }
+    __device__ __forceinline__ void add(float x) {
+        float e, f;
+        s = two_sum(s, x, e);
+        c = two_sum(c, e, f);
+        d = __fadd_rn(d, f);
+    }
+    __device__ __forceinline__ void add_product(float x, float y) {
+        const float hi = __fmul_rn(x, y), lo = __fmaf_rn(x, y, -hi);
+        float e, f, g;
+        s = two_sum(s, hi, e);
+        e = two_sum(lo, e, f);
+        c = two_sum(c, e, g);
+        d = __fadd_rn(d, __fadd_rn(f, g));
+    }
+    __device__ __forceinline__ double value() const { return ((double)d + (double)c) + (double)s; }
+};
+
+// Sums of rho, rho u_x, rho u_y and rho u_z (0 when dim = 2) over initial fields: the total
+// mass and momentum of the equilibrium state built from them (relation (rhoq) summed over the
+// lattice; sum_j v_j f_eq,j = rho u at every node). rho may be NULL (rho = 1).
+//
+// FP64 issues at 2 operations per clock per SM on this GPU: three conversions and three
+// additions per node in FP64 took 195 us at 4096^2, for 201 MB of fields. ExactSum does the
+// same in some 60 FP32 operations per node, under the time of the loads, with a smaller
+// error, and is added to FP64 every 32 nodes. The last block to finish adds the blocks'
+// partials in a fixed order (a second kernel cost 6 us), and leaves *ticket at 0 again.
+template <int NV>
+__global__ void __launch_bounds__(kReduceThreads, kReduceMinBlocks)
+    k_mean_flow(Fields fld, int64_t n, int dim, double* __restrict__ part,
+                unsigned* __restrict__ ticket, double* __restrict__ out) {
+    constexpr int kRunPacks = 32 / NV;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    const int64_t packs = n / NV, stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    while (i < packs) {
+        ExactSum run[4];
+        for (int t = 0; t < kRunPacks && i < packs; ++t, i += stride) {
+            float r[NV], u[3][NV];
+            load_field<NV>(fld.rho, i, 1.0f, r);
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                if (a < dim) load_field<NV>(fld.u[a], i, 0.0f, u[a]);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                run[0].add(r[k]);
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    if (a < dim) run[1 + a].add_product(r[k], u[a][k]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] += run[c].value();
+    }
+    block_sum4<kReduceThreads>(v, part + 4 * (int64_t)blockIdx.x);
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();  // the partials before the ticket
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double w[4] = {0.0, 0.0, 0.0, 0.0};
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) w[c] += __ldcg(part + 4 * b + c);
+    }
+    block_sum4<kReduceThreads>(w, out);
+    if (threadIdx.x == 0) *ticket = 0u;
+}
+
+// The same sums with FP64 arithmetic throughout, for fields whose FP32 products leave the
+// range of FP32 (the host falls back to it).
 __global__ void __launch_bounds__(kReduceThreads) k_mean_flow_partial(
-    const float* __restrict__ rho, const float* __restrict__ u, int64_t n, int64_t plane,
-    int dim, double* __restrict__ part) {
+    Fields fld, int64_t n, int dim, double* __restrict__ part) {
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const double r = rho ? (double)rho[i] : 1.0;
+        const double r = fld.rho ? (double)fld.rho[i] : 1.0;
         v[0] += r;
-        v[1] += r * (double)u[i];
-        v[2] += r * (double)u[plane + i];
-        if (dim == 3) v[3] += r * (double)u[2 * plane + i];
+        v[1] += r * (double)fld.u[0][i];
+        v[2] += r * (double)fld.u[1][i];
+        if (dim == 3) v[3] += r * (double)fld.u[2][i];
     }
     block_sum4<kReduceThreads>(v, part + 4 * (int64_t)blockIdx.x);
 }
@@ -607,62 +697,60 @@ cudaError_t launch_step_conserved(int storage, int um, int nv, const void* src, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_init_eq(int storage, void* dst, const float* rho, const float* u, int64_t n,
-                           const StoreRef& rho_ref, float inv_lambda, cudaStream_t st,
-                           int basis) {
-    const int g = grid_stride_blocks(n, 256);
-    if (basis == 1) {
-        switch (storage) {
-            case kStoreF32:
-                k_init_eq_product<float><<<g, 256, 0, st>>>(static_cast<float*>(dst), rho, u, n,
-                                                            rho_ref, inv_lambda);
-                break;
-            case kStoreF16:
-                k_init_eq_product<__half><<<g, 256, 0, st>>>(static_cast<__half*>(dst), rho, u, n,
-                                                             rho_ref, inv_lambda);
-                break;
-            case kStoreBF16:
-                k_init_eq_product<__nv_bfloat16><<<g, 256, 0, st>>>(
-                    static_cast<__nv_bfloat16*>(dst), rho, u, n, rho_ref, inv_lambda);
-                break;
-            default: return cudaErrorInvalidValue;
-        }
-        return cudaGetLastError();
-    }
-    switch (storage) {
-        case kStoreF32:
-            k_init_eq<float><<<g, 256, 0, st>>>(static_cast<float*>(dst), rho, u, n, rho_ref,
-                                                inv_lambda);
-            break;
-        case kStoreF16:
-            k_init_eq<__half><<<g, 256, 0, st>>>(static_cast<__half*>(dst), rho, u, n, rho_ref,
-                                                 inv_lambda);
-            break;
-        case kStoreBF16:
-            k_init_eq<__nv_bfloat16><<<g, 256, 0, st>>>(static_cast<__nv_bfloat16*>(dst), rho, u,
-                                                        n, rho_ref, inv_lambda);
-            break;
+namespace {
+
+// Four nodes per thread where n and every pointer allow one vector access per plane.
+bool fields_vec4(const Fields& f, int dim, int64_t n) {
+    uintptr_t bits = reinterpret_cast<uintptr_t>(f.rho);
+    for (int a = 0; a < dim; ++a) bits |= reinterpret_cast<uintptr_t>(f.u[a]);
+    return n % 4 == 0 && bits % 16 == 0;
+}
+
+template <typename T, int BASIS>
+void init_eq_t(void* dst, const Fields& f, int64_t n, const StoreRef& ref, float inv_lambda,
+               cudaStream_t st) {
+    if (fields_vec4(f, 2, n))
+        k_init_eq<T, BASIS, 4><<<grid_stride_blocks(n / 4, 256), 256, 0, st>>>(
+            static_cast<T*>(dst), f, n, ref, inv_lambda);
+    else
+        k_init_eq<T, BASIS, 1><<<grid_stride_blocks(n, 256), 256, 0, st>>>(
+            static_cast<T*>(dst), f, n, ref, inv_lambda);
+}
+
+template <typename T>
+void moments_t(const void* src, float* rho, float* u, int64_t n, const StoreRef& ref,
+               float lambda, cudaStream_t st) {
+    const uintptr_t bits = reinterpret_cast<uintptr_t>(rho) | reinterpret_cast<uintptr_t>(u);
+    if (n % 4 == 0 && bits % 16 == 0)
+        k_moments<T, 4><<<grid_stride_blocks(n / 4, 256), 256, 0, st>>>(
+            static_cast<const T*>(src), rho, u, n, ref, lambda);
+    else
+        k_moments<T, 1><<<grid_stride_blocks(n, 256), 256, 0, st>>>(
+            static_cast<const T*>(src), rho, u, n, ref, lambda);
+}
+
+}  // namespace
+
+cudaError_t launch_init_eq(int storage, void* dst, const Fields& f, int64_t n,
+                           const StoreRef& ref, float inv_lambda, cudaStream_t st, int basis) {
+    switch (storage * 2 + (basis != 0)) {
+        case 0: init_eq_t<float, 0>(dst, f, n, ref, inv_lambda, st); break;
+        case 1: init_eq_t<float, 1>(dst, f, n, ref, inv_lambda, st); break;
+        case 2: init_eq_t<__half, 0>(dst, f, n, ref, inv_lambda, st); break;
+        case 3: init_eq_t<__half, 1>(dst, f, n, ref, inv_lambda, st); break;
+        case 4: init_eq_t<__nv_bfloat16, 0>(dst, f, n, ref, inv_lambda, st); break;
+        case 5: init_eq_t<__nv_bfloat16, 1>(dst, f, n, ref, inv_lambda, st); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_moments(int storage, const void* src, float* rho, float* u, int64_t n,
-                           const StoreRef& rho_ref, float lambda, cudaStream_t st) {
-    const int g = grid_stride_blocks(n, 256);
+                           const StoreRef& ref, float lambda, cudaStream_t st) {
     switch (storage) {
-        case kStoreF32:
-            k_moments<float><<<g, 256, 0, st>>>(static_cast<const float*>(src), rho, u, n,
-                                                rho_ref, lambda);
-            break;
-        case kStoreF16:
-            k_moments<__half><<<g, 256, 0, st>>>(static_cast<const __half*>(src), rho, u, n,
-                                                 rho_ref, lambda);
-            break;
-        case kStoreBF16:
-            k_moments<__nv_bfloat16><<<g, 256, 0, st>>>(
-                static_cast<const __nv_bfloat16*>(src), rho, u, n, rho_ref, lambda);
-            break;
+        case kStoreF32: moments_t<float>(src, rho, u, n, ref, lambda, st); break;
+        case kStoreF16: moments_t<__half>(src, rho, u, n, ref, lambda, st); break;
+        case kStoreBF16: moments_t<__nv_bfloat16>(src, rho, u, n, ref, lambda, st); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -685,9 +773,21 @@ int conserved_blocks(int64_t n) {
     return (int)(b < 1 ? 1 : (b > full ? full : b));
 }
 
-cudaError_t launch_mean_flow(const float* rho, const float* u, int64_t n, int64_t plane,
-                             int dim, double* partials, int nblk, double* out, cudaStream_t st) {
-    k_mean_flow_partial<<<nblk, kReduceThreads, 0, st>>>(rho, u, n, plane, dim, partials);
+cudaError_t launch_mean_flow(const Fields& f, int64_t n, int dim, double* partials, int nblk,
+                             unsigned* ticket, double* out, cudaStream_t st) {
+    const int nv = fields_vec4(f, dim, n) ? 4 : 1;
+    const int64_t need = (n / nv + kReduceThreads - 1) / kReduceThreads;
+    const int blocks = (int)(need < 1 ? 1 : (need < nblk ? need : nblk));
+    if (nv == 4)
+        k_mean_flow<4><<<blocks, kReduceThreads, 0, st>>>(f, n, dim, partials, ticket, out);
+    else
+        k_mean_flow<1><<<blocks, kReduceThreads, 0, st>>>(f, n, dim, partials, ticket, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mean_flow_fp64(const Fields& f, int64_t n, int dim, double* partials,
+                                  int nblk, double* out, cudaStream_t st) {
+    k_mean_flow_partial<<<nblk, kReduceThreads, 0, st>>>(f, n, dim, partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_conserved_final<<<1, kReduceThreads, 0, st>>>(partials, nblk, 0.0, 0.0, 0.0, 1.0, out);

@@ -728,45 +728,65 @@ __constant__ int kC3X[19] = {0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0
 __constant__ int kC3Y[19] = {0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 0, 0, 1, -1, 1, -1};
 __constant__ int kC3Z[19] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1};
 
-// g_j = f_eq,j(rho, u) - f_eq,j(rho_ref, U), difference form as in the D2Q9 kernel.
-template <typename T>
-__global__ void k_init_eq3(T* __restrict__ dst, const float* __restrict__ rho,
-                           const float* __restrict__ u, int64_t n, StoreRef3 ref,
-                           float inv_lambda) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+// g_j = f_eq,j(rho, u) - f_eq,j(rho_ref, U), difference form as in the D2Q9 kernel; NV
+// consecutive nodes per thread.
+template <typename T, int NV>
+__global__ void __launch_bounds__(256)
+    k_init_eq3(T* __restrict__ dst, Fields fld, int64_t n, StoreRef3 ref, float inv_lambda) {
+    const int64_t packs = n / NV;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < packs;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const float r = rho ? rho[i] : 1.0f;
-        const float ux = u[i] * inv_lambda, uy = u[n + i] * inv_lambda, uz = u[2 * n + i] * inv_lambda;
-        const float uu = ux * ux + uy * uy + uz * uz;
-        const float UU = ref.ux * ref.ux + ref.uy * ref.uy + ref.uz * ref.uz;
+        float r[NV], v[3][NV];
+        load_field<NV>(fld.rho, i, 1.0f, r);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) load_field<NV>(fld.u[a], i, 0.0f, v[a]);
 #pragma unroll
         for (int j = 0; j < 19; ++j) {
             const float cx = (float)kC3X[j], cy = (float)kC3Y[j], cz = (float)kC3Z[j];
-            const float cu = cx * ux + cy * uy + cz * uz;
-            const float cU = cx * ref.ux + cy * ref.uy + cz * ref.uz;
             const float w = wgt3(j);
-            const float pu = 3.0f * cu + 4.5f * cu * cu - 1.5f * uu;
-            const float pU = 3.0f * cU + 4.5f * cU * cU - 1.5f * UU;
-            dst[j * n + i] = from_f<T>(w * (r - ref.rho) + w * (r * pu - ref.rho * pU));
+            float g[NV];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                const float ux = v[0][k] * inv_lambda, uy = v[1][k] * inv_lambda,
+                            uz = v[2][k] * inv_lambda;
+                const float uu = ux * ux + uy * uy + uz * uz;
+                const float UU = ref.ux * ref.ux + ref.uy * ref.uy + ref.uz * ref.uz;
+                const float cu = cx * ux + cy * uy + cz * uz;
+                const float cU = cx * ref.ux + cy * ref.uy + cz * ref.uz;
+                const float pu = 3.0f * cu + 4.5f * cu * cu - 1.5f * uu;
+                const float pU = 3.0f * cU + 4.5f * cU * cU - 1.5f * UU;
+                g[k] = w * (r[k] - ref.rho) + w * (r[k] * pu - ref.rho * pU);
+            }
+            store_pack<T, NV>(dst + j * n + i * NV, g);
         }
     }
 }
 
-template <typename T>
-__global__ void k_moments3(const T* __restrict__ src, float* __restrict__ rho,
-                           float* __restrict__ u, int64_t n, StoreRef3 ref, float lambda) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+template <typename T, int NV>
+__global__ void __launch_bounds__(256)
+    k_moments3(const T* __restrict__ src, float* __restrict__ rho, float* __restrict__ u,
+               int64_t n, StoreRef3 ref, float lambda) {
+    const int64_t packs = n / NV;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < packs;
          i += (int64_t)gridDim.x * blockDim.x) {
-        float g[19];
+        float g[19][NV], r[NV], v[3][NV];
 #pragma unroll
-        for (int j = 0; j < 19; ++j) g[j] = to_f(src[j * n + i]);
-        const NodeMoments3 m = node_moments3(g);
-        const float r = ref.rho + m.drho;
-        if (rho) rho[i] = r;
+        for (int j = 0; j < 19; ++j) load_pack<T, NV>(src + j * n + i * NV, true, g[j]);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            float h[19];
+#pragma unroll
+            for (int j = 0; j < 19; ++j) h[j] = g[j][k];
+            const NodeMoments3 m = node_moments3(h);
+            r[k] = ref.rho + m.drho;
+            v[0][k] = lambda * (ref.jx + m.jx) / r[k];
+            v[1][k] = lambda * (ref.jy + m.jy) / r[k];
+            v[2][k] = lambda * (ref.jz + m.jz) / r[k];
+        }
+        if (rho) store_pack<float, NV>(rho + i * NV, r);
         if (u) {
-            u[i] = lambda * (ref.jx + m.jx) / r;
-            u[n + i] = lambda * (ref.jy + m.jy) / r;
-            u[2 * n + i] = lambda * (ref.jz + m.jz) / r;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) store_pack<float, NV>(u + a * n + i * NV, v[a]);
         }
     }
 }
@@ -1119,20 +1139,43 @@ cudaError_t launch_step3(int storage, int um, int nv, const void* src, void* dst
     }
 }
 
-cudaError_t launch_init_eq3(int storage, void* dst, const float* rho, const float* u, int64_t n,
+namespace {
+
+template <typename T>
+void init_eq3_t(void* dst, const Fields& f, int64_t n, const StoreRef3& ref, float inv_lambda,
+                cudaStream_t st) {
+    uintptr_t bits = reinterpret_cast<uintptr_t>(f.rho);
+    for (int a = 0; a < 3; ++a) bits |= reinterpret_cast<uintptr_t>(f.u[a]);
+    if (n % 4 == 0 && bits % 16 == 0)
+        k_init_eq3<T, 4><<<grid_stride_blocks(n / 4, 256), 256, 0, st>>>(static_cast<T*>(dst), f,
+                                                                         n, ref, inv_lambda);
+    else
+        k_init_eq3<T, 1><<<grid_stride_blocks(n, 256), 256, 0, st>>>(static_cast<T*>(dst), f, n,
+                                                                     ref, inv_lambda);
+}
+
+// Packs of 8 bytes in FP32 and 16-bit storage (wider packs of 19 planes spill).
+template <typename T>
+void moments3_t(const void* src, float* rho, float* u, int64_t n, const StoreRef3& ref,
+                float lambda, cudaStream_t st) {
+    constexpr int NV = 8 / (int)sizeof(T);
+    const uintptr_t bits = reinterpret_cast<uintptr_t>(rho) | reinterpret_cast<uintptr_t>(u);
+    if (n % NV == 0 && bits % 16 == 0)
+        k_moments3<T, NV><<<grid_stride_blocks(n / NV, 256), 256, 0, st>>>(
+            static_cast<const T*>(src), rho, u, n, ref, lambda);
+    else
+        k_moments3<T, 1><<<grid_stride_blocks(n, 256), 256, 0, st>>>(static_cast<const T*>(src),
+                                                                     rho, u, n, ref, lambda);
+}
+
+}  // namespace
+
+cudaError_t launch_init_eq3(int storage, void* dst, const Fields& f, int64_t n,
                             const StoreRef3& ref, float inv_lambda, cudaStream_t st) {
-    const int g = grid_stride_blocks(n, 256);
     switch (storage) {
-        case kStoreF32:
-            k_init_eq3<float><<<g, 256, 0, st>>>(static_cast<float*>(dst), rho, u, n, ref, inv_lambda);
-            break;
-        case kStoreF16:
-            k_init_eq3<__half><<<g, 256, 0, st>>>(static_cast<__half*>(dst), rho, u, n, ref, inv_lambda);
-            break;
-        case kStoreBF16:
-            k_init_eq3<__nv_bfloat16><<<g, 256, 0, st>>>(static_cast<__nv_bfloat16*>(dst), rho, u, n,
-                                                        ref, inv_lambda);
-            break;
+        case kStoreF32: init_eq3_t<float>(dst, f, n, ref, inv_lambda, st); break;
+        case kStoreF16: init_eq3_t<__half>(dst, f, n, ref, inv_lambda, st); break;
+        case kStoreBF16: init_eq3_t<__nv_bfloat16>(dst, f, n, ref, inv_lambda, st); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -1140,18 +1183,10 @@ cudaError_t launch_init_eq3(int storage, void* dst, const float* rho, const floa
 
 cudaError_t launch_moments3(int storage, const void* src, float* rho, float* u, int64_t n,
                             const StoreRef3& ref, float lambda, cudaStream_t st) {
-    const int g = grid_stride_blocks(n, 256);
     switch (storage) {
-        case kStoreF32:
-            k_moments3<float><<<g, 256, 0, st>>>(static_cast<const float*>(src), rho, u, n, ref, lambda);
-            break;
-        case kStoreF16:
-            k_moments3<__half><<<g, 256, 0, st>>>(static_cast<const __half*>(src), rho, u, n, ref, lambda);
-            break;
-        case kStoreBF16:
-            k_moments3<__nv_bfloat16><<<g, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(src), rho, u,
-                                                        n, ref, lambda);
-            break;
+        case kStoreF32: moments3_t<float>(src, rho, u, n, ref, lambda, st); break;
+        case kStoreF16: moments3_t<__half>(src, rho, u, n, ref, lambda, st); break;
+        case kStoreBF16: moments3_t<__nv_bfloat16>(src, rho, u, n, ref, lambda, st); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -41,7 +41,7 @@ struct lbmrv_s {
     int64_t tile_n = 0;   // the step count and mode that `tile` was planned for
     int tile_um = -1;
     lbmrv::TilePlan tile;
-    double* red = nullptr;   // reduction scratch: 8 * red_blocks partials + 8 results
+    double* red = nullptr;   // reduction scratch: 8 * red_blocks partials + 8 results + ticket
     int red_blocks = 0;
     double* fused = nullptr;  // partials of the step with fused sums, + 4 results (lazy)
     int64_t fused_doubles = 0;
@@ -206,6 +206,10 @@ inline int kernel_mode(const lbmrv_s* h) {
     if (h->umode == LBMRV_UT_FLUID) return UM_FLUID;
     return h->ut0 ? UM_FIELD : UM_ANALYTIC;
 }
+
+// Sums {rho, rho u_x, rho u_y, rho u_z} of n nodes of initial fields, read back (synchronises
+// the handle's stream).
+cudaError_t flow_sums(const lbmrv_s* h, const Fields& f, int64_t n, double sums[4]);
 
 // Widest usable pack for the fused step on buffers a, b (1: one node per thread).
 int choose_width(const lbmrv_s* h, const void* a, const void* b);

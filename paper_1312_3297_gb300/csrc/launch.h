@@ -79,7 +79,13 @@ cudaError_t launch_step_conserved(int storage, int um, int nv, const void* src, 
                                   double jx_ref, double jy_ref, double lambda,
                                   double* partials, double* out);
 
-cudaError_t launch_init_eq(int storage, void* dst, const float* rho, const float* u, int64_t n,
+// Initial fields: density (or null: 1) and velocity components, n floats each.
+struct Fields {
+    const float* rho = nullptr;
+    const float* u[3] = {nullptr, nullptr, nullptr};
+};
+
+cudaError_t launch_init_eq(int storage, void* dst, const Fields& f, int64_t n,
                            const StoreRef& ref, float inv_lambda, cudaStream_t st,
                            int basis = 0);
 
@@ -95,16 +101,20 @@ cudaError_t launch_conserved(int storage, const void* src, int64_t n, int64_t pl
                              double rho_ref, double jx_ref, double jy_ref, double lambda,
                              double* partials, int nblk, double* out, cudaStream_t st);
 
-// Sums {rho, rho u_x, rho u_y, rho u_z} over nodes 0 .. n-1 of initial fields (rho NULL:
-// 1; u: dim planes `plane` floats apart) into out[4] (device); partials: 4 * nblk doubles.
-cudaError_t launch_mean_flow(const float* rho, const float* u, int64_t n, int64_t plane,
-                             int dim, double* partials, int nblk, double* out, cudaStream_t st);
+// Sums {rho, rho u_x, rho u_y, rho u_z} over nodes 0 .. n-1 of initial fields into out[4]
+// (device); partials: 4 * nblk doubles; ticket: a device word that is 0 between calls. FP32
+// arithmetic with the rounding errors carried along, for densities and momenta well inside the
+// range of FP32; _fp64 for any.
+cudaError_t launch_mean_flow(const Fields& f, int64_t n, int dim, double* partials, int nblk,
+                             unsigned* ticket, double* out, cudaStream_t st);
+cudaError_t launch_mean_flow_fp64(const Fields& f, int64_t n, int dim, double* partials,
+                                  int nblk, double* out, cudaStream_t st);
 
 // ---------------------------------------------------------------- D3Q19
 int step3_vector_width(int storage, int nx);
 cudaError_t launch_step3(int storage, int um, int nv, const void* src, void* dst,
                          const StepArgs3& a, cudaStream_t st);
-cudaError_t launch_init_eq3(int storage, void* dst, const float* rho, const float* u, int64_t n,
+cudaError_t launch_init_eq3(int storage, void* dst, const Fields& f, int64_t n,
                             const StoreRef3& ref, float inv_lambda, cudaStream_t st);
 cudaError_t launch_moments3(int storage, const void* src, float* rho, float* u, int64_t n,
                             const StoreRef3& ref, float lambda, cudaStream_t st);

@@ -53,24 +53,41 @@ void warn_rates(lbmrv_t h, int lattice, const double* s, const char* who) {
 }
 }  // namespace
 
+cudaError_t flow_sums(const lbmrv_s* h, const Fields& f, int64_t n, double sums[4]) {
+    double* res = h->red + 8 * (size_t)h->red_blocks;
+    for (int c = 0; c < 4; ++c) sums[c] = 0.0;
+    auto read = [&](cudaError_t e) {
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(sums, res, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
+        return e == cudaSuccess ? cudaStreamSynchronize(h->stream) : e;
+    };
+    cudaError_t e = read(launch_mean_flow(f, n, h->dim, h->red, h->red_blocks,
+                                          reinterpret_cast<unsigned*>(res + 8), res, h->stream));
+    if (e != cudaSuccess) return e;
+    // densities far from 1, or momenta beyond FP32: the FP64 kernel
+    const double mean = sums[0] / (double)n;
+    const bool usual = std::isfinite(sums[0]) && std::isfinite(sums[1]) &&
+                       std::isfinite(sums[2]) && std::isfinite(sums[3]) && mean > 1e-6 &&
+                       mean < 1e6;
+    if (usual) return cudaSuccess;
+    return read(launch_mean_flow_fp64(f, n, h->dim, h->red, h->red_blocks, res, h->stream));
+}
+
+namespace {
+
 // The automatic reference velocity: U_ref = sum rho u / sum rho over the fields an
-// equilibrium is about to be built from (an FP64 device reduction, read back on the host).
+// equilibrium is about to be built from (a device reduction, read back on the host).
 // Total mass and momentum are invariants of the periodic scheme (relation (rhoq) summed
 // over the lattice: relaxation conserves them at every node, transport moves them), so
 // U_ref stays the mean flow of the whole run. Synchronises the handle's stream.
-int apply_auto_reference(lbmrv_t h, const float* rho, const float* u, const char* who) {
+int apply_auto_reference(lbmrv_t h, const Fields& f, const char* who) {
     if (!h->ref_auto) return LBMRV_OK;
     if (h->slab)
         return fail(h, LBMRV_E_INVAL,
                     "%s: a slab needs the reference shared by all slabs (lbmrv_set_reference)",
                     who);
-    double* res = h->red + 8 * (size_t)h->red_blocks;
-    double sums[4] = {0.0, 0.0, 0.0, 0.0};
-    cudaError_t e = launch_mean_flow(rho, u, h->n, h->n, h->dim, h->red, h->red_blocks, res,
-                                     h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(sums, res, sizeof(sums), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    double sums[4];
+    cudaError_t e = flow_sums(h, f, h->n, sums);
     if (e != cudaSuccess) return cuda_fail(h, e, who);
     for (int c = 0; c < 4; ++c)
         if (!std::isfinite(sums[c]))
@@ -80,6 +97,32 @@ int apply_auto_reference(lbmrv_t h, const float* rho, const float* u, const char
     for (int a = 0; a < 3; ++a) h->u_ref[a] = a < h->dim ? sums[1 + a] / sums[0] : 0.0;
     return LBMRV_OK;
 }
+
+// The equilibrium of the fields into the current state, time 0.
+int init_from_fields(lbmrv_t h, const Fields& f, const char* who) {
+    int rc = apply_auto_reference(h, f, who);
+    if (rc != LBMRV_OK) return rc;
+    cudaError_t e;
+    if (h->dim == 2)
+        e = launch_init_eq(h->storage, h->f[h->cur], f, h->n, store_ref(h),
+                           (float)(1.0 / h->lambda), h->stream, h->basis);
+    else
+        e = launch_init_eq3(h->storage, h->f[h->cur], f, h->n, store_ref3(h),
+                            (float)(1.0 / h->lambda), h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, who);
+    h->t = 0;
+    return LBMRV_OK;
+}
+
+// rho and d planes of n velocity values, as in lbmrv_init_equilibrium.
+Fields planes(const lbmrv_s* h, const float* rho, const float* u) {
+    Fields f;
+    f.rho = rho;
+    for (int a = 0; a < h->dim; ++a) f.u[a] = u + a * h->n;
+    return f;
+}
+
+}  // namespace
 
 int fail(lbmrv_t h, int code, const char* fmt, ...) {
     char* buf = h ? h->err : g_create_err;
@@ -192,7 +235,9 @@ int lbmrv_create(lbmrv_t* out, int lattice, const int64_t dims[3], double lambda
         ok = cudaMalloc(&h->f[0], bytes) == cudaSuccess && cudaMalloc(&h->f[1], bytes) == cudaSuccess;
     }
     h->red_blocks = conserved_blocks(h->n);
-    ok = ok && cudaMalloc(&h->red, sizeof(double) * (8 * (size_t)h->red_blocks + 8)) == cudaSuccess;
+    ok = ok && cudaMalloc(&h->red, sizeof(double) * (8 * (size_t)h->red_blocks + 9)) == cudaSuccess;
+    // the reduction's ticket; done when the blocking copy below is
+    ok = ok && cudaMemset(h->red + 8 * (size_t)h->red_blocks + 8, 0, sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc(&h->sin_x, sizeof(float) * (size_t)h->nx) == cudaSuccess;
     if (ok) {
         std::vector<float> tab((size_t)h->nx);
@@ -316,18 +361,22 @@ int lbmrv_init_equilibrium(lbmrv_t h, const float* rho_dev, const float* u_dev) 
     if (!h) return fail(nullptr, LBMRV_E_INVAL, "lbmrv_init_equilibrium: NULL handle");
     if (!u_dev) return fail(h, LBMRV_E_INVAL, "lbmrv_init_equilibrium: u is NULL");
     DeviceGuard g(h->device);
-    int rc = apply_auto_reference(h, rho_dev, u_dev, "lbmrv_init_equilibrium");
-    if (rc != LBMRV_OK) return rc;
-    cudaError_t e;
-    if (h->dim == 2)
-        e = launch_init_eq(h->storage, h->f[h->cur], rho_dev, u_dev, h->n, store_ref(h),
-                           (float)(1.0 / h->lambda), h->stream, h->basis);
-    else
-        e = launch_init_eq3(h->storage, h->f[h->cur], rho_dev, u_dev, h->n, store_ref3(h),
-                            (float)(1.0 / h->lambda), h->stream);
-    if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_init_equilibrium");
-    h->t = 0;
-    return LBMRV_OK;
+    return init_from_fields(h, planes(h, rho_dev, u_dev), "lbmrv_init_equilibrium");
+}
+
+int lbmrv_init_equilibrium_fields(lbmrv_t h, const float* rho_dev, const float* ux_dev,
+                                  const float* uy_dev, const float* uz_dev) {
+    const char* who = "lbmrv_init_equilibrium_fields";
+    if (!h) return fail(nullptr, LBMRV_E_INVAL, "%s: NULL handle", who);
+    if (!ux_dev || !uy_dev || (h->dim == 3 && !uz_dev))
+        return fail(h, LBMRV_E_INVAL, "%s: a velocity component is NULL", who);
+    DeviceGuard g(h->device);
+    Fields f;
+    f.rho = rho_dev;
+    f.u[0] = ux_dev;
+    f.u[1] = uy_dev;
+    if (h->dim == 3) f.u[2] = uz_dev;
+    return init_from_fields(h, f, who);
 }
 
 int lbmrv_init_equilibrium_host(lbmrv_t h, const float* rho_host, const float* u_host) {
@@ -342,18 +391,8 @@ int lbmrv_init_equilibrium_host(lbmrv_t h, const float* rho_host, const float* u
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(stage + h->n, u_host, h->dim * nb, cudaMemcpyHostToDevice, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_init_equilibrium_host: copy");
-    const float* rho = rho_host ? stage : nullptr;
-    int rc = apply_auto_reference(h, rho, stage + h->n, "lbmrv_init_equilibrium_host");
-    if (rc != LBMRV_OK) return rc;
-    if (h->dim == 2)
-        e = launch_init_eq(h->storage, h->f[h->cur], rho, stage + h->n, h->n, store_ref(h),
-                           (float)(1.0 / h->lambda), h->stream, h->basis);
-    else
-        e = launch_init_eq3(h->storage, h->f[h->cur], rho, stage + h->n, h->n, store_ref3(h),
-                            (float)(1.0 / h->lambda), h->stream);
-    if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_init_equilibrium_host");
-    h->t = 0;
-    return LBMRV_OK;
+    return init_from_fields(h, planes(h, rho_host ? stage : nullptr, stage + h->n),
+                            "lbmrv_init_equilibrium_host");
 }
 
 int lbmrv_step(lbmrv_t h, int64_t n) {

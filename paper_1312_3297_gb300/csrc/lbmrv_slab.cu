@@ -262,13 +262,11 @@ int lbmrv_flow_sums(lbmrv_t h, const float* rho_dev, const float* u_dev, double 
     if (!u_dev || !out_host) return fail(h, LBMRV_E_INVAL, "lbmrv_flow_sums: NULL argument");
     DeviceGuard g(h->device);
     const int64_t o = owned_first(h);
-    double* res = h->red + 8 * (size_t)h->red_blocks;
-    double sums[4] = {0.0, 0.0, 0.0, 0.0};
-    cudaError_t e = launch_mean_flow(rho_dev ? rho_dev + o : nullptr, u_dev + o, owned_count(h),
-                                     h->n, h->dim, h->red, h->red_blocks, res, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(sums, res, sizeof(sums), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    Fields f;
+    f.rho = rho_dev ? rho_dev + o : nullptr;
+    for (int a = 0; a < h->dim; ++a) f.u[a] = u_dev + a * h->n + o;
+    double sums[4];
+    const cudaError_t e = flow_sums(h, f, owned_count(h), sums);
     if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_flow_sums");
     for (int c = 0; c < 4; ++c) out_host[c] = sums[c];
     return LBMRV_OK;

@@ -100,6 +100,18 @@ __device__ __forceinline__ void load_pack(const T* __restrict__ p, bool act, flo
     }
 }
 
+// Pack i of an FP32 field, or `absent` everywhere where there is no field.
+template <int NV>
+__device__ __forceinline__ void load_field(const float* __restrict__ p, int64_t i, float absent,
+                                           float out[NV]) {
+    if (p) {
+        load_pack<float, NV>(p + i * NV, true, out);
+    } else {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) out[k] = absent;
+    }
+}
+
 // Row segment starting one element left of the pack: (prev, v0, ..., v_{NV-2}).
 template <typename T, int NV>
 __device__ __forceinline__ void load_from_left(const T* __restrict__ row, int x0, int xprev,

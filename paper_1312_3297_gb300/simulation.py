@@ -68,6 +68,9 @@ class D2Q9:
         self.dtype = STORAGE_DTYPES[self.storage]
 
     # -- stream order between torch's current stream and the handle's stream
+    def _on_current_stream(self) -> bool:
+        return torch.cuda.current_stream(self.device) == self.stream
+
     def _sync_in(self):
         """The handle's stream waits for work already queued on torch's current stream
         (inputs that torch produced)."""
@@ -140,10 +143,14 @@ class D2Q9:
         if len(u_components) != self.DIM:
             raise ValueError(f"expected {self.DIM} velocity components")
         rho = torch.as_tensor(rho, dtype=torch.float32, device=self.device).contiguous()
-        u = torch.stack([torch.as_tensor(c, dtype=torch.float32, device=self.device)
-                         for c in u_components]).contiguous()
-        self._sync_in()
-        B.lbmrv_init_equilibrium(self.h, rho, u)
+        u = [torch.as_tensor(c, dtype=torch.float32, device=self.device) for c in u_components]
+        if self._on_current_stream() and all(c.shape == u[0].shape for c in u):
+            u = [c.contiguous() for c in u]
+            B.lbmrv_init_equilibrium_fields(self.h, rho, *u)
+        else:  # read on another stream: a copy that the caller's tensors do not share
+            u = torch.stack(u).contiguous()
+            self._sync_in()
+            B.lbmrv_init_equilibrium(self.h, rho, u)
         self._keep = (rho, u)  # the copy is asynchronous on the stream
 
     def init_equilibrium_host(self, rho_host, u_host):
