@@ -111,6 +111,8 @@ def library_path() -> str:
 def load(build_if_needed: bool = True) -> ctypes.CDLL:
     """Load liblbmrv.so (building it first when stale). Raises if it cannot."""
     global _lib
+    if _lib is not None:  # set once, under the lock
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.build() if build_if_needed else _build.LIB_PATH

@@ -56,6 +56,8 @@ class D2Q9:
         self._bufs = [torch.empty(nbytes, dtype=torch.uint8, device=self.device)
                       for _ in range(2)]
         self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
+        self._index = (self.device.index if self.device.index is not None
+                       else torch.cuda.current_device())
         with torch.cuda.device(self.device):
             self.h = B.lbmrv_create(self.LATTICE, dims, self.lam, list(s), self.mode,
                                     self.storage, self.rho_ref, self.stream,
@@ -69,21 +71,21 @@ class D2Q9:
 
     # -- stream order between torch's current stream and the handle's stream
     def _on_current_stream(self) -> bool:
-        return torch.cuda.current_stream(self.device) == self.stream
+        # by raw handle: torch.cuda.current_stream builds a Stream object on every call
+        mine = self.stream if isinstance(self.stream, int) else self.stream.cuda_stream
+        return torch._C._cuda_getCurrentRawStream(self._index) == mine
 
     def _sync_in(self):
         """The handle's stream waits for work already queued on torch's current stream
         (inputs that torch produced)."""
-        cur = torch.cuda.current_stream(self.device)
-        if isinstance(self.stream, torch.cuda.Stream) and cur != self.stream:
-            self.stream.wait_stream(cur)
+        if not self._on_current_stream() and isinstance(self.stream, torch.cuda.Stream):
+            self.stream.wait_stream(torch.cuda.current_stream(self.device))
 
     def _sync_out(self):
         """Torch's current stream waits for the handle's queued work (outputs torch will
         read)."""
-        cur = torch.cuda.current_stream(self.device)
-        if isinstance(self.stream, torch.cuda.Stream) and cur != self.stream:
-            cur.wait_stream(self.stream)
+        if not self._on_current_stream() and isinstance(self.stream, torch.cuda.Stream):
+            torch.cuda.current_stream(self.device).wait_stream(self.stream)
 
     # -- lifecycle
     def close(self):
@@ -170,7 +172,7 @@ class D2Q9:
         u = torch.empty((self.DIM,) + self.shape, dtype=torch.float32, device=self.device)
         B.lbmrv_moments(self.h, rho, u)
         self._sync_out()
-        return (rho,) + tuple(u[a] for a in range(self.DIM))
+        return (rho,) + u.unbind(0)
 
     def moments_host(self, rho_host=None, u_host=None):
         if rho_host is None:
