@@ -32,19 +32,36 @@
 namespace lbmrv {
 namespace {
 
-// Warps per block, on neighbouring strips of the same rows (measured: FP32 4096^2 204 k MLUPS
-// with two against 201 k with one; 16-bit 8192^2 227 k with one against 221 k with two).
-template <typename T>
-constexpr int kWarps = sizeof(T) == 4 ? 2 : 1;
-template <typename T>
-constexpr int kThreads = 32 * kWarps<T>;
 constexpr int kLevels = kMarchSteps;
 constexpr int kNV = 4;  // nodes per pack
 // Packs of a strip that are stored: each level loses one node at both ends of a strip, whose
 // neighbours belong to the next strips, so lanes 0 and 31 are recomputed there (kLevels <= kNV
 // + 1 keeps the loss within those lanes).
 constexpr int kUse = 30;
-constexpr int64_t kMarchMinBytes = 128 << 20;  // about the L2 (129 MB)
+
+// Strips of a row: one if the row has no more packs than a warp has lanes (its lanes are then
+// each other's periodic neighbours and nothing is recomputed), else of kUse packs. Warps per
+// block, on neighbouring strips of the same rows: two in FP32 unless that leaves a good part of
+// them idle (4096^2 204 k MLUPS with two, 201 k with one), one in 16-bit storage (8192^2 227 k
+// with one, 221 k with two).
+struct Strips {
+    int packs, warps, groups, segs;
+    Strips(int storage, int nx, int ny, int64_t resident_warps) {
+        packs = nx / kNV;
+        const int strips = packs <= 32 ? 1 : (packs + kUse - 1) / kUse;
+        warps = storage == kStoreF32 && (strips % 2 == 0 || strips > 8) ? 2 : 1;
+        groups = (strips + warps - 1) / warps;
+        // One segment of rows per resident block and strip group. Segments under 8 rows repeat
+        // too many relaxations (2 (kLevels - 1) rows each): half as many then (FP32 1536 x 1000
+        // 145 k MLUPS against 138 k). Long 16-bit segments are halved, so that blocks that end
+        // early leave work to take (8192^2 227 k against 224 k; no gain in FP32).
+        int64_t s = resident_warps / warps / groups;
+        if (s * 8 > ny) s = resident_warps / 2 / warps / groups;
+        if (storage != kStoreF32 && s * 64 < ny) s = 2 * s;
+        if (s > ny) s = ny;
+        segs = (int)(s < 1 ? 1 : s);
+    }
+};
 
 // A pack in storage form: NV consecutive nodes in W 32-bit words.
 template <typename T>
@@ -74,9 +91,9 @@ __device__ __forceinline__ void put_pair(uint32_t* w, int k, F2 v) {
 
 // (prev, v0, ..., v_{NV-2}), prev from the left lane.
 template <typename T>
-__device__ __forceinline__ void from_left(uint32_t v[kW<T>]) {
+__device__ __forceinline__ void from_left(uint32_t v[kW<T>], int left) {
     constexpr int W = kW<T>;
-    const uint32_t p = __shfl_up_sync(kFullMask, v[W - 1], 1);
+    const uint32_t p = __shfl_sync(kFullMask, v[W - 1], left);
 #pragma unroll
     for (int i = W - 1; i >= 0; --i) {
         const uint32_t l = i ? v[i - 1] : p;
@@ -85,9 +102,9 @@ __device__ __forceinline__ void from_left(uint32_t v[kW<T>]) {
 }
 // (v1, ..., v_{NV-1}, next), next from the right lane.
 template <typename T>
-__device__ __forceinline__ void from_right(uint32_t v[kW<T>]) {
+__device__ __forceinline__ void from_right(uint32_t v[kW<T>], int right) {
     constexpr int W = kW<T>;
-    const uint32_t p = __shfl_down_sync(kFullMask, v[0], 1);
+    const uint32_t p = __shfl_sync(kFullMask, v[0], right);
 #pragma unroll
     for (int i = 0; i < W; ++i) {
         const uint32_t r = i < W - 1 ? v[i + 1] : p;
@@ -96,13 +113,13 @@ __device__ __forceinline__ void from_right(uint32_t v[kW<T>]) {
 }
 
 template <typename T>
-__device__ __forceinline__ void shift_x(uint32_t g[9][kW<T>]) {
-    from_left<T>(g[1]);
-    from_right<T>(g[3]);
-    from_left<T>(g[5]);
-    from_right<T>(g[6]);
-    from_right<T>(g[7]);
-    from_left<T>(g[8]);
+__device__ __forceinline__ void shift_x(uint32_t g[9][kW<T>], int left, int right) {
+    from_left<T>(g[1], left);
+    from_right<T>(g[3], right);
+    from_left<T>(g[5], left);
+    from_right<T>(g[6], right);
+    from_right<T>(g[7], right);
+    from_left<T>(g[8], left);
 }
 
 template <int W>
@@ -153,30 +170,39 @@ __device__ __forceinline__ void relax_pack(uint32_t g[9][kW<T>], float amp, cons
 
 // Shared memory, private to each thread: the next row's nine packs, and nine packs of delay
 // line per level but the last; a stored field adds its next row's two packs.
-template <typename T>
-constexpr int kSlot = kThreads<T> * 4 * kW<T>;
-template <typename T, int UM>
-constexpr int kSmem = kSlot<T> * 9 * kLevels + (UM == UM_FIELD ? 2 * kThreads<T> * 16 : 0);
+template <typename T, int WPB>
+constexpr int kSlot = 32 * WPB * 4 * kW<T>;
+template <typename T, int UM, int WPB>
+constexpr int kSmem = kSlot<T, WPB> * 9 * kLevels + (UM == UM_FIELD ? 2 * 32 * WPB * 16 : 0);
 // 16 warps per SM (128 registers, no spills); 12 with a stored field, whose rows of the three
 // levels stay in registers.
-template <typename T, int UM>
-constexpr int kBlocks = (UM == UM_FIELD ? 12 : 16) / kWarps<T>;
+template <int UM>
+constexpr int kSmWarps = UM == UM_FIELD ? 12 : 16;
 
-template <typename T, int UM, int BASIS, int RCP>
-__global__ void __launch_bounds__(kThreads<T>, (kBlocks<T, UM>))
+template <typename T, int UM, int BASIS, int RCP, int WPB>
+__global__ void __launch_bounds__(32 * WPB, kSmWarps<UM> / WPB)
     k_march3(const T* __restrict__ src, T* __restrict__ dst, StepArgs a, MarchAmps amps,
              int groups, int segs) {
     extern __shared__ __align__(16) char smem[];
     pdl_wait_prior();
     pdl_allow_next();
-    constexpr int W = kW<T>, SB = kSlot<T>;
+    constexpr int W = kW<T>, SB = kSlot<T, WPB>, NT = 32 * WPB;
     const int nx = a.nx, ny = a.ny;
     const int64_t n = (int64_t)nx * ny;
     const int lane = threadIdx.x & 31;
     const int grp = blockIdx.x % groups, seg = blockIdx.x / groups;
     const int packs = nx / kNV;
-    const int pk = (grp * kWarps<T> + (threadIdx.x >> 5)) * kUse + lane - 1;
-    const bool act = lane >= 1 && lane <= kUse && pk < packs;
+    int pk, left = lane - 1, right = lane + 1;  // this lane's pack, the neighbours' lanes
+    bool act;
+    if (packs <= 32) {
+        pk = lane;
+        act = lane < packs;
+        if (lane == 0) left = packs - 1;
+        if (lane == packs - 1) right = 0;
+    } else {
+        pk = (grp * WPB + (threadIdx.x >> 5)) * kUse + lane - 1;
+        act = lane >= 1 && lane <= kUse && pk < packs;
+    }
     int pw = pk % packs;  // lanes past the row's ends take its periodic continuation
     if (pw < 0) pw += packs;
     const int x0 = pw * kNV;
@@ -196,7 +222,7 @@ __global__ void __launch_bounds__(kThreads<T>, (kBlocks<T, UM>))
         }
         if constexpr (UM == UM_FIELD) {
             cp_async16(field, a.ut0 + o0 + x0);
-            cp_async16(field + kThreads<T> * 16, a.ut0 + n + o0 + x0);
+            cp_async16(field + NT * 16, a.ut0 + n + o0 + x0);
         }
         cp_async_commit();
     };
@@ -235,9 +261,9 @@ __global__ void __launch_bounds__(kThreads<T>, (kBlocks<T, UM>))
                 }
             }
             ldw<kNV>(field, reinterpret_cast<uint32_t*>(bx[0]));
-            ldw<kNV>(field + kThreads<T> * 16, reinterpret_cast<uint32_t*>(by[0]));
+            ldw<kNV>(field + NT * 16, reinterpret_cast<uint32_t*>(by[0]));
         }
-        shift_x<T>(g);
+        shift_x<T>(g, left, right);
         relax_pack<T, UM, BASIS, RCP>(g, amps.v[0], bx[0], by[0], a);
         // the slots have been read: fetch the next row behind levels 2 and 3
         if (i + 1 < rows) load_row((int64_t)r * nx, (int64_t)rp * nx, (int64_t)rq * nx);
@@ -246,7 +272,7 @@ __global__ void __launch_bounds__(kThreads<T>, (kBlocks<T, UM>))
             if (i < 2 * (l - 1)) continue;
             // the row below: {0,1,3} as level l left them one row ago, {2,5,6} two rows ago
             // (a ring of two), {4,7,8} now
-            shift_x<T>(g);
+            shift_x<T>(g, left, right);
             char* const d = mine + 9 * l * SB;
             char* const e = d + (3 + 3 * (i & 1)) * SB;
             constexpr int c0[3] = {0, 1, 3}, cp[3] = {2, 5, 6};
@@ -286,29 +312,30 @@ __global__ void __launch_bounds__(kThreads<T>, (kBlocks<T, UM>))
     }
 }
 
+template <typename T, int UM, int BASIS, int RCP, int WPB>
+cudaError_t launch_w(const void* src, void* dst, const StepArgs& a, const MarchAmps& amps,
+                     const Strips& p, cudaStream_t st) {
+    auto kernel = k_march3<T, UM, BASIS, RCP, WPB>;
+    constexpr int smem = kSmem<T, UM, WPB>;
+    static std::atomic<int> resident[kMaxDevicesOcc];  // sets the kernel's shared memory, once
+    int full = 0;
+    cudaError_t e = resident_blocks(kernel, resident, 32 * WPB, smem, 32, &full);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl_smem(kernel, dim3((unsigned)((int64_t)p.groups * p.segs)), dim3(32 * WPB), smem,
+                        st, static_cast<const T*>(src), static_cast<T*>(dst), a, amps, p.groups,
+                        p.segs);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <typename T, int UM, int BASIS, int RCP>
 cudaError_t launch_t(const void* src, void* dst, const StepArgs& a, const MarchAmps& amps,
                      cudaStream_t st) {
-    const int packs = a.nx / kNV;
-    const int groups = (packs + kWarps<T> * kUse - 1) / (kWarps<T> * kUse);
-    auto kernel = k_march3<T, UM, BASIS, RCP>;
-    static std::atomic<int> resident[kMaxDevicesOcc];
-    int full = 0;
-    cudaError_t e = resident_blocks(kernel, resident, kThreads<T>, kSmem<T, UM>, 32, &full);
-    if (e != cudaSuccess) return e;
-    // One segment of rows per resident block and strip group. Segments under 8 rows repeat too
-    // many relaxations (2 (kLevels - 1) rows each): half as many then (FP32 1536 x 1000 145 k
-    // MLUPS against 138 k). Long 16-bit segments are halved, so that blocks that end early leave
-    // work to take (8192^2 227 k against 224 k; no gain in FP32).
-    int64_t segs = full / groups;
-    if (segs * 8 > a.ny) segs = full / 2 / groups;
-    if (sizeof(T) == 2 && segs * 64 < a.ny) segs = 2 * segs;
-    if (segs > a.ny) segs = a.ny;
-    if (segs < 1) segs = 1;
-    e = launch_pdl_smem(kernel, dim3((unsigned)(groups * segs)), dim3(kThreads<T>), kSmem<T, UM>, st,
-                        static_cast<const T*>(src), static_cast<T*>(dst), a, amps, groups,
-                        (int)segs);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    const Strips p(sizeof(T) == 4 ? kStoreF32 : kStoreF16, a.nx, a.ny,
+                   (int64_t)kSmWarps<UM> * sm_count());
+    if constexpr (sizeof(T) == 4) {
+        if (p.warps == 2) return launch_w<T, UM, BASIS, RCP, 2>(src, dst, a, amps, p, st);
+    }
+    return launch_w<T, UM, BASIS, RCP, 1>(src, dst, a, amps, p, st);
 }
 
 // 1/rho in the form that the one-step kernel of the same rows uses (d2q9_kernels.cu), so that
@@ -351,20 +378,28 @@ cudaError_t launch_basis(int um, const void* s, void* d, const StepArgs& a,
 
 }  // namespace
 
-bool march_usable(int storage, int um, int basis, int nx, int ny, const void* a, const void* b,
-                  const float* ut0) {
+double march_step_us(int storage, int um, int basis, int nx, int ny, const void* a,
+                     const void* b, const float* ut0) {
     const int bytes = storage == kStoreF32 ? 16 : 8;
     if (nx % kNV != 0 || reinterpret_cast<uintptr_t>(a) % bytes != 0 ||
         reinterpret_cast<uintptr_t>(b) % bytes != 0)
-        return false;
+        return 1e30;
     if (um == UM_FIELD && (reinterpret_cast<uintptr_t>(ut0) % 16 != 0 ||
                            (storage != kStoreF32 && basis == 1 && nx % 8 != 0)))
-        return false;
-    // While both states stay in L2 a single step is not bound by DRAM and the repeated
-    // relaxations cost more than the traffic saved: FP32 1024^2 (75 MB of states) 124 k MLUPS
-    // either way, 1448^2 (151 MB) 88 k -> 141 k; 16-bit 1024 x 2048 (75 MB) 198 k against 169 k
-    // here, 2048^2 (151 MB) 165 k -> 182 k.
-    return 2 * 9 * (int64_t)nx * ny * (storage == kStoreF32 ? 4 : 2) > kMarchMinBytes;
+        return 1e30;
+    // Measured on GB300: 0.235 nodes per ns and lane in use with every warp resident, 0.205
+    // with half of them, 6 rows repeated in three per segment, a third of a launch.
+    const int64_t warps = (int64_t)(um == UM_FIELD ? 12 : 16) * sm_count();
+    const Strips p(storage, nx, ny, warps);
+    const double useful = (double)p.packs / (32.0 * p.groups * p.warps);
+    const double rows = (double)ny / p.segs;
+    const bool half = (int64_t)p.groups * p.warps * p.segs * 3 < warps * 2;
+    // the correctly rounded 1/rho is slower, the more so with few warps to hide it
+    const bool rn = um != UM_ZERO && (storage == kStoreF32 ? basis == 1
+                                                           : basis == 0 && nx % 8 != 0);
+    const double rate = (half ? 205.0 : 235.0) * (um == UM_FIELD ? 0.82 : 1.0) *
+                        (!rn ? 1.0 : half && storage != kStoreF32 ? 0.7 : 0.9);
+    return (double)nx * ny / (rate * 1e3 * useful) * (1.0 + 2.0 / rows) + 0.7;
 }
 
 cudaError_t launch_march(int storage, int um, const void* src, void* dst, const StepArgs& a,

@@ -14,27 +14,50 @@ constexpr double kSerial = 2.0;      // loads and stores of a tile that nothing 
 
 bool fits_l2(double nodes, int node_bytes) { return 2.0 * node_bytes * nodes < 128e6; }
 
-// A single-step launch: the launch and the time per million nodes at its pack width, with the
-// states in L2 or in DRAM.
-double single_step_us(int storage, int nv, double nodes, int node_bytes) {
-    const bool l2 = fits_l2(nodes, node_bytes);
-    double per_m;
-    if (storage == kStoreF32)
-        per_m = nv == 4 ? (l2 ? 6.4 : 10.5) : nv == 2 ? (l2 ? 8.2 : 10.9) : (l2 ? 7.7 : 11.2);
-    else
-        per_m = nv == 8 ? (l2 ? 4.4 : 5.8) : nv == 4 ? 6.7 : nv == 2 ? 7.7 : 9.5;
-    return 1.9 + per_m * 1e-6 * nodes;
-}
+}  // namespace
 
 int sm_count() {
+    static std::atomic<int> sms_of[kMaxDevicesOcc];
     int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        return 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kMaxDevicesOcc) return 152;
+    sms = sms_of[dev].load(std::memory_order_relaxed);
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            sms < 1)
+            return 152;
+        sms_of[dev].store(sms, std::memory_order_relaxed);
+    }
     return sms;
 }
 
-}  // namespace
+// The launch, and the time per million nodes at the pack width nv: with the states in L2, too
+// large for it, or between; more where a row leaves many of a block's 128 threads without a
+// pack.
+double single_step_us(int storage, int um, int nv, int nx, int ny) {
+    const double nodes = (double)nx * ny;
+    const bool f32 = storage == kStoreF32;
+    const double field = um == UM_FIELD ? 8.0 : 0.0;
+    const double both = (2.0 * 9.0 * (f32 ? 4 : 2) + field) * nodes;
+    const bool l2 = both < 78e6, dram = both > 128e6;
+    double per_m;
+    if (f32)
+        per_m = nv == 4 ? (l2 ? 6.4 : dram ? 10.5 : 7.8)
+              : nv == 2 ? (dram ? 10.9 : 8.2)
+                        : (dram ? 11.2 : 7.7);
+    else
+        per_m = nv == 8 ? (dram ? 5.8 : 4.4) : nv == 4 ? 5.4 : nv == 2 ? 7.7 : 9.5;
+    if (nv >= 4) {
+        const int span = 128 * nv;
+        const double used = (double)nx / (span * ((nx + span - 1) / span));
+        if (f32)
+            per_m *= used < 0.1 ? 0.3 / used : 1.0 + 0.2 * (1.0 - used);
+        else
+            per_m *= used < 0.4 ? 0.5 / used : 1.0 + 0.8 * (1.0 - used);
+    }
+    if (um == UM_ZERO && !f32 && !dram) per_m *= 0.87;
+    if (um == UM_FIELD) per_m *= !dram || f32 ? 1.07 : 1.22;
+    return 1.9 + per_m * 1e-6 * nodes;
+}
 
 // The plan with the least modelled time for n steps: steps per pass, array size and warps per
 // block. Small lattices take many steps per pass (64^2: 10, over 32 x 22 arrays), since a launch
@@ -50,9 +73,12 @@ TilePlan tile_plan(int storage, int um, int nv, int nx, int ny, int64_t n) {
     const int elem = storage == kStoreF32 ? 4 : 2, sms = sm_count();
     const double nodes = (double)nx * ny;
     const bool in_l2 = fits_l2(nodes, 9 * elem);
-    const double per_sm = kItem / sms;
+    // the correctly rounded 1/rho of 16-bit storage, and the conversions, take a little longer
+    const double item_us = kItem * (elem == 2 && um != UM_ZERO ? (nv == 8 ? 1.03 : 1.1) : 1.0);
+    const double per_sm = item_us / sms;
     // only where clearly less than single steps
-    double least = 0.93 * n * single_step_us(storage, nv, nodes, 9 * elem);
+    double least = 0.93 * n * single_step_us(storage, um, nv, nx, ny);
+    best.us = n * single_step_us(storage, um, nv, nx, ny);
     // likely lengths first: a good plan early drops most of the others unevaluated
     constexpr int lengths[] = {5, 10, 4, 3, 8, 6, 12, 2};
     constexpr int heights[] = {12, 16, 20, 22, 24, 26, 28, 32, 36, 38, 40, 44, 46, 48, 56, 62};
@@ -95,7 +121,7 @@ TilePlan tile_plan(int storage, int um, int nv, int nx, int ny, int64_t n) {
                     auto wave = [&](int resident) {
                         const double busy = (double)resident * warps;
                         const double item =
-                            kItem * (busy < 20.0 ? 1.0 + 0.03 * (20.0 - busy) : 1.0);
+                            item_us * (busy < 20.0 ? 1.0 + 0.03 * (20.0 - busy) : 1.0);
                         double us = 0.0;
                         for (int k = 0; k < s; ++k) {
                             const int pairs = rx / 32 * ((ry - k - 1) / 2 - k / 2 + 1);
@@ -112,12 +138,15 @@ TilePlan tile_plan(int storage, int um, int nv, int nx, int ny, int64_t n) {
                     if (fit == 1 && tiles > sms) us += kSerial * (tiles - sms) / sms;
                     const double total = m * (kLaunch + us);
                     if (total < least) {
-                        least = total;
+                        least = best.us = total;
                         best.steps = s;
                         best.rx = rx;
                         best.ry = ry;
                         best.warps = warps;
                         best.launches = m;
+                        best.per_sm = full == 0 || rest == 0 && full == 1
+                                          ? (tiles + sms - 1) / sms
+                                          : 0;
                     }
                 }
             }

@@ -38,8 +38,10 @@ struct lbmrv_s {
     int64_t t = 0;
     const float* ut0 = nullptr;
     double amp = 0.0, period = 0.0;
-    int64_t tile_n = 0;   // the step count and mode that `tile` was planned for
-    int tile_um = -1;
+    // how lbmrv_step takes plan_n steps in mode plan_um (D2Q9, automatic kernel variant)
+    int64_t plan_n = 0;
+    int plan_um = -1;
+    bool march = false;
     lbmrv::TilePlan tile;
     double* red = nullptr;   // reduction scratch: 8 * red_blocks partials + 8 results + ticket
     int red_blocks = 0;

@@ -32,15 +32,22 @@ int step_vector_width(int storage, int nx);
 cudaError_t launch_step(int storage, int um, int nv, const void* src, void* dst,
                         const StepArgs& a, cudaStream_t st, int basis = 0);
 
+// SMs of the current device (152 if the runtime does not say).
+int sm_count();
+
+// Modelled times of one step in microseconds, for the choice between the forms of the D2Q9
+// step: one launch per step at pack width nv; one of launch_march's three (1e30 where it does
+// not suit the lattice: row length, alignment; ut0 the stored field, or null).
+double single_step_us(int storage, int um, int nv, int nx, int ny);
+double march_step_us(int storage, int um, int basis, int nx, int ny, const void* a,
+                     const void* b, const float* ut0);
+
 // kMarchSteps steps src -> dst in one pass over memory (d2q9_march.cu), the bits of that many
 // launch_step calls. a: the arguments of the first of them; amps: amp_t of each.
-// march_usable: whether the lattice suits it (u~0 the stored field, or null).
 constexpr int kMarchSteps = 3;
 struct MarchAmps {
     float v[kMarchSteps];
 };
-bool march_usable(int storage, int um, int basis, int nx, int ny, const void* a, const void* b,
-                  const float* ut0);
 cudaError_t launch_march(int storage, int um, const void* src, void* dst, const StepArgs& a,
                          const MarchAmps& amps, cudaStream_t st, int basis);
 
@@ -56,7 +63,9 @@ struct TileAmps {
 struct TilePlan {
     int steps = 1;  // 1: single-step launches are faster
     int rx = 0, ry = 0, warps = 0;
+    int per_sm = 0;  // blocks per SM if that makes one wave (else 0: as many as fit)
     int64_t launches = 0;  // for the n steps planned: `launches` passes of at most `steps`
+    double us = 0.0;       // modelled time of the n steps
 };
 inline int64_t tile_bytes(int rx, int ry, int elem, int um) {
     return 9LL * rx * (ry + 3) * elem +

@@ -352,6 +352,7 @@ int lbmrv_set_utilde(lbmrv_t h, const float* ut0_dev, double amplitude, double p
     if (h->lattice == LBMRV_D3Q19 && h->umode == LBMRV_UT_PRESCRIBED && !ut0_dev)
         return fail(h, LBMRV_E_UNSUPPORTED, "lbmrv_set_utilde: D3Q19 needs a u~0 field");
     h->ut0 = ut0_dev;
+    h->plan_n = 0;  // the choice of a step's form depends on the field's alignment
     h->amp = amplitude;
     h->period = period;
     return LBMRV_OK;
@@ -395,6 +396,21 @@ int lbmrv_init_equilibrium_host(lbmrv_t h, const float* rho_host, const float* u
                             "lbmrv_init_equilibrium_host");
 }
 
+// Which form of the D2Q9 step takes n steps in least time; kept for the next call of as many.
+static void plan_steps(lbmrv_t h, int nv, int um, int64_t n) {
+    if (h->plan_n == n && h->plan_um == um) return;
+    const int nx = (int)h->nx, ny = (int)h->ny;
+    const double march = march_step_us(h->storage, um, h->basis, nx, ny, h->f[0], h->f[1], h->ut0);
+    const double single = single_step_us(h->storage, um, nv, nx, ny);
+    h->tile = TilePlan();
+    h->tile.us = n * single;
+    if (n >= kTileMinSteps) h->tile = tile_plan(h->storage, um, nv, nx, ny, n);
+    const int64_t rest = n % kMarchSteps;
+    h->march = (n - rest) * march + rest * single < 0.95 * h->tile.us;
+    h->plan_n = n;
+    h->plan_um = um;
+}
+
 int lbmrv_step(lbmrv_t h, int64_t n) {
     lbmrv::TraceRange trace("lbmrv_step");
     if (!h) return fail(nullptr, LBMRV_E_INVAL, "lbmrv_step: NULL handle");
@@ -404,34 +420,23 @@ int lbmrv_step(lbmrv_t h, int64_t n) {
     DeviceGuard g(h->device);
     const int nv = choose_width(h, h->f[0], h->f[1]);
     int64_t k = 0;
-    // passes of kMarchSteps steps; an odd number of steps per pass leaves every state in the
-    // buffer that as many single steps would leave it in
-    if (h->dim == 2 && h->width == 0 && !h->slab && n >= kMarchSteps &&
-        march_usable(h->storage, kernel_mode(h), h->basis, (int)h->nx, (int)h->ny, h->f[0],
-                     h->f[1], h->ut0)) {
-        for (; n - k >= kMarchSteps; k += kMarchSteps) {
+    if (n >= kMarchSteps && h->dim == 2 && h->width == 0 && !h->slab) {
+        const int um = kernel_mode(h);
+        plan_steps(h, nv, um, n);
+        // passes of kMarchSteps steps; an odd number of steps per pass leaves every state in
+        // the buffer that as many single steps would leave it in
+        for (; h->march && n - k >= kMarchSteps; k += kMarchSteps) {
             MarchAmps amps;
-            for (int l = 0; l < kMarchSteps; ++l)
-                amps.v[l] = prescribed_amp(h, h->t + 1 + l);
-            cudaError_t e = launch_march(h->storage, kernel_mode(h), h->f[h->cur],
-                                         h->f[1 - h->cur], make_args(h, h->t + 1), amps,
-                                         h->stream, h->basis);
+            for (int l = 0; l < kMarchSteps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);
+            cudaError_t e = launch_march(h->storage, um, h->f[h->cur], h->f[1 - h->cur],
+                                         make_args(h, h->t + 1), amps, h->stream, h->basis);
             if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step");
             h->cur = 1 - h->cur;
             h->t += kMarchSteps;
         }
-    }
-    // passes over shared-memory tiles, where they are faster than single steps; of equal
-    // lengths to within one
-    if (k == 0 && n >= kTileMinSteps && h->dim == 2 && h->width == 0 && !h->slab) {
-        const int um = kernel_mode(h);
-        if (h->tile_n != n || h->tile_um != um) {
-            h->tile = tile_plan(h->storage, um, nv, (int)h->nx, (int)h->ny, n);
-            h->tile_n = n;
-            h->tile_um = um;
-        }
+        // passes over shared-memory tiles, of equal lengths to within one
         TilePlan p = h->tile;
-        for (int64_t m = p.launches; m > 0; --m) {
+        for (int64_t m = h->march ? 0 : p.launches; m > 0; --m) {
             p.steps = (int)((n - k + m - 1) / m);
             TileAmps amps;
             for (int l = 0; l < p.steps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);

@@ -45,10 +45,10 @@ def assert_same_as_single_steps(cls, nx, ny, mode, storage, steps):
             many.state_ptr() == many._bufs[0].data_ptr())
 
 
-# rows of one pack; a row of exactly 15 strips of 30 packs, of one pack more and one fewer;
+# rows of one pack; of 31, 32 and 33 packs (one periodic strip up to 32); a row of exactly 15 strips of 30 packs, of one pack more and one fewer;
 # fewer rows than segments; a 16-bit row that 8-node packs do not divide (2052, 1804); 4.2 M
 # nodes put both states of every storage type beyond L2
-SIZES = [(4, 900001), (1800, 2003), (1804, 2001), (1796, 2003), (131072, 28), (2052, 1801)]
+SIZES = [(4, 900001), (128, 25000), (132, 25000), (124, 25001), (1800, 2003), (1804, 2001), (1796, 2003), (131072, 28), (2052, 1801)]
 
 
 @pytest.mark.parametrize("storage", ["fp32", "fp16", "bf16"])
