@@ -216,8 +216,11 @@ class D2Q9:
         return B.lbmrv_state_ptr(self.h)
 
     # -- adjoint (FP32 storage)
+    def adjoint_workspace_bytes(self, n: int, seg: int) -> int:
+        return B.lbmrv_adjoint_workspace_bytes(self.h, n, seg)
+
     def adjoint_workspace(self, n: int, seg: int) -> torch.Tensor:
-        nbytes = B.lbmrv_adjoint_workspace_bytes(self.h, n, seg)
+        nbytes = self.adjoint_workspace_bytes(n, seg)
         if nbytes <= 0:
             raise ValueError(f"invalid adjoint window n={n}, seg={seg}")
         return torch.empty(nbytes, dtype=torch.uint8, device=self.device)
