@@ -91,6 +91,28 @@ __device__ __forceinline__ void block_sum4(double v[4], double* out) {
     }
 }
 
+// Whether the calling block is the last of nblk to get here; its partial results are then, and
+// those of all the others, visible to it. thread 0 has written the block's own.
+__device__ __forceinline__ bool last_block(unsigned* ticket, unsigned nblk) {
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();  // the partials before the ticket
+        last = atomicAdd(ticket, 1u) == nblk - 1;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Where the step with fused sums leaves them: 4 doubles per block, and the totals with the
+// reference state's added.
+struct StepSums {
+    double* part;
+    unsigned* ticket;  // 0 between launches
+    double* out;
+    double rho_n, jx_n, jy_n, lambda;
+};
+
 template <typename T, int UM, int BASIS>
 __global__ void __launch_bounds__(256) k_step_scalar(const T* __restrict__ src,
                                                      T* __restrict__ dst, StepArgs a) {
@@ -162,8 +184,7 @@ constexpr int step_vec_min_blocks =
 
 template <typename T, int NV, int UM, int BASIS, bool SUMS = false>
 __global__ void __launch_bounds__(128, (step_vec_min_blocks<T, BASIS, NV, UM, SUMS>))
-    k_step_vec(const T* __restrict__ src, T* __restrict__ dst, StepArgs a,
-               double* __restrict__ part) {
+    k_step_vec(const T* __restrict__ src, T* __restrict__ dst, StepArgs a, StepSums sums_out) {
     pdl_wait_prior();
     pdl_allow_next();
     const int nx = a.nx, ny = a.ny;
@@ -276,7 +297,31 @@ __global__ void __launch_bounds__(128, (step_vec_min_blocks<T, BASIS, NV, UM, SU
 #pragma unroll
         for (int c = 0; c < 3; ++c) v[c] = sums[c] + (double)run_r[c];
         v[3] = (double)bad;
-        block_sum4<128>(v, part + 4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x));
+        const StepSums& o = sums_out;
+        block_sum4<128>(v, o.part + 4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x));
+        // The last block to finish adds the slots, in a fixed order, and leaves *ticket at 0
+        // again (two more launches took 11 us for this).
+        const int nblk = gridDim.x * gridDim.y;
+        if (!last_block(o.ticket, nblk)) return;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = 0.0;
+        for (int b = threadIdx.x; b < nblk; b += 128) {
+            const double2 p0 = __ldcg(reinterpret_cast<const double2*>(o.part + 4 * b));
+            const double2 p1 = __ldcg(reinterpret_cast<const double2*>(o.part + 4 * b + 2));
+            v[0] += p0.x;
+            v[1] += p0.y;
+            v[2] += p1.x;
+            v[3] += p1.y;
+        }
+        __shared__ double res[4];
+        block_sum4<128>(v, res);
+        if (threadIdx.x == 0) {
+            o.out[0] = res[0] + o.rho_n;
+            o.out[1] = o.lambda * (res[1] + o.jx_n);
+            o.out[2] = o.lambda * (res[2] + o.jy_n);
+            o.out[3] = res[3];
+            *o.ticket = 0u;
+        }
     }
 }
 
@@ -497,14 +542,7 @@ __global__ void __launch_bounds__(kReduceThreads, kReduceMinBlocks)
         for (int c = 0; c < 4; ++c) v[c] += run[c].value();
     }
     block_sum4<kReduceThreads>(v, part + 4 * (int64_t)blockIdx.x);
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        __threadfence();  // the partials before the ticket
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
+    if (!last_block(ticket, gridDim.x)) return;
     double w[4] = {0.0, 0.0, 0.0, 0.0};
     for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
 #pragma unroll
@@ -530,32 +568,17 @@ __global__ void __launch_bounds__(kReduceThreads) k_mean_flow_partial(
     block_sum4<kReduceThreads>(v, part + 4 * (int64_t)blockIdx.x);
 }
 
-// Block b adds partials [256 b, 256 b + 256) of 4 doubles each into out[4 b].
-__global__ void __launch_bounds__(kReduceThreads) k_sum_partials(const double* __restrict__ part,
-                                                                 int64_t nblk,
-                                                                 double* __restrict__ out) {
-    const int64_t i = (int64_t)blockIdx.x * kReduceThreads + threadIdx.x;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    if (i < nblk) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = part[4 * i + c];
-    }
-    block_sum4<kReduceThreads>(v, out + 4 * (int64_t)blockIdx.x);
-}
-
-
-// With the sums (part != nullptr) the grid has as many blocks as are resident at once
-// (rows strided over blocks), and *nblk receives the number of block slots written: with
-// one row per block the FP64 block reductions of a 4096^2 step took longer than the step.
+// With the sums the grid has as many blocks as are resident at once (rows strided over blocks):
+// with one row per block the FP64 block reductions of a 4096^2 step took longer than the step.
 template <typename T, int NV, int UM, int BASIS>
-cudaError_t launch_vec(const T* s, T* d, const StepArgs& a, cudaStream_t st, double* part,
-                       int64_t* nblk) {
+cudaError_t launch_vec(const T* s, T* d, const StepArgs& a, cudaStream_t st,
+                       const StepSums* sums) {
     const int gx = ((a.nx / NV) + 127) / 128;
     const int rows = a.ny < 65535 ? a.ny : 65535;
     // successive steps overlap their launch with the previous step's tail (pdl.cuh)
-    if (!part)
+    if (!sums)
         return launch_pdl(k_step_vec<T, NV, UM, BASIS, false>, dim3(gx, rows), dim3(128), st, s,
-                          d, a, static_cast<double*>(nullptr));
+                          d, a, StepSums{});
     auto kernel = k_step_vec<T, NV, UM, BASIS, true>;
     static std::atomic<int> resident[kMaxDevicesOcc];
     int full = 0;
@@ -563,28 +586,27 @@ cudaError_t launch_vec(const T* s, T* d, const StepArgs& a, cudaStream_t st, dou
     if (e != cudaSuccess) return e;
     const int per_x = full / gx;
     const int gy = per_x < 1 ? 1 : (per_x < rows ? per_x : rows);
-    if (nblk) *nblk = (int64_t)gx * gy;
-    return launch_pdl(kernel, dim3(gx, gy), dim3(128), st, s, d, a, part);
+    return launch_pdl(kernel, dim3(gx, gy), dim3(128), st, s, d, a, *sums);
 }
 
 template <typename T, int UM, int BASIS>
 cudaError_t step_dispatch_nv(const void* src, void* dst, const StepArgs& a, cudaStream_t st,
-                             int nv, double* part, int64_t* nblk) {
+                             int nv, const StepSums* sums) {
     const T* s = static_cast<const T*>(src);
     T* d = static_cast<T*>(dst);
     const int gy = a.ny < 65535 ? a.ny : 65535;
     cudaError_t e;
     if (nv == 1) {
-        if (part) return cudaErrorInvalidValue;  // sums are fused into the vector kernel only
+        if (sums) return cudaErrorInvalidValue;  // sums are fused into the vector kernel only
         e = launch_pdl(k_step_scalar<T, UM, BASIS>, dim3((a.nx + 255) / 256, gy), dim3(256), st,
                        s, d, a);
     } else if (nv == 2) {
-        e = launch_vec<T, 2, UM, BASIS>(s, d, a, st, part, nblk);
+        e = launch_vec<T, 2, UM, BASIS>(s, d, a, st, sums);
     } else if (nv == 4) {
-        e = launch_vec<T, 4, UM, BASIS>(s, d, a, st, part, nblk);
+        e = launch_vec<T, 4, UM, BASIS>(s, d, a, st, sums);
     } else if (nv == 8) {
         if constexpr (sizeof(T) == 2) {
-            e = launch_vec<T, 8, UM, BASIS>(s, d, a, st, part, nblk);
+            e = launch_vec<T, 8, UM, BASIS>(s, d, a, st, sums);
         } else {
             return cudaErrorInvalidValue;
         }
@@ -596,25 +618,25 @@ cudaError_t step_dispatch_nv(const void* src, void* dst, const StepArgs& a, cuda
 
 template <typename T, int BASIS>
 cudaError_t step_dispatch_um(const void* src, void* dst, const StepArgs& a, cudaStream_t st,
-                             int um, int nv, double* part, int64_t* nblk) {
+                             int um, int nv, const StepSums* sums) {
     switch (um) {
         case UM_ZERO:
-            return step_dispatch_nv<T, UM_ZERO, BASIS>(src, dst, a, st, nv, part, nblk);
+            return step_dispatch_nv<T, UM_ZERO, BASIS>(src, dst, a, st, nv, sums);
         case UM_FLUID:
-            return step_dispatch_nv<T, UM_FLUID, BASIS>(src, dst, a, st, nv, part, nblk);
+            return step_dispatch_nv<T, UM_FLUID, BASIS>(src, dst, a, st, nv, sums);
         case UM_ANALYTIC:
-            return step_dispatch_nv<T, UM_ANALYTIC, BASIS>(src, dst, a, st, nv, part, nblk);
+            return step_dispatch_nv<T, UM_ANALYTIC, BASIS>(src, dst, a, st, nv, sums);
         case UM_FIELD:
-            return step_dispatch_nv<T, UM_FIELD, BASIS>(src, dst, a, st, nv, part, nblk);
+            return step_dispatch_nv<T, UM_FIELD, BASIS>(src, dst, a, st, nv, sums);
         default: return cudaErrorInvalidValue;
     }
 }
 
 template <typename T>
 cudaError_t step_dispatch_basis(const void* src, void* dst, const StepArgs& a, cudaStream_t st,
-                                int um, int nv, int basis, double* part, int64_t* nblk) {
-    return basis == 0 ? step_dispatch_um<T, 0>(src, dst, a, st, um, nv, part, nblk)
-                      : step_dispatch_um<T, 1>(src, dst, a, st, um, nv, part, nblk);
+                                int um, int nv, int basis, const StepSums* sums) {
+    return basis == 0 ? step_dispatch_um<T, 0>(src, dst, a, st, um, nv, sums)
+                      : step_dispatch_um<T, 1>(src, dst, a, st, um, nv, sums);
 }
 
 }  // namespace
@@ -647,16 +669,14 @@ int step_vector_width(int storage, int nx) {
 namespace {
 
 cudaError_t step_storage(int storage, int um, int nv, const void* src, void* dst,
-                         const StepArgs& a, cudaStream_t st, int basis, double* part,
-                         int64_t* nblk = nullptr) {
+                         const StepArgs& a, cudaStream_t st, int basis, const StepSums* sums) {
     switch (storage) {
         case kStoreF32:
-            return step_dispatch_basis<float>(src, dst, a, st, um, nv, basis, part, nblk);
+            return step_dispatch_basis<float>(src, dst, a, st, um, nv, basis, sums);
         case kStoreF16:
-            return step_dispatch_basis<__half>(src, dst, a, st, um, nv, basis, part, nblk);
+            return step_dispatch_basis<__half>(src, dst, a, st, um, nv, basis, sums);
         case kStoreBF16:
-            return step_dispatch_basis<__nv_bfloat16>(src, dst, a, st, um, nv, basis, part,
-                                                      nblk);
+            return step_dispatch_basis<__nv_bfloat16>(src, dst, a, st, um, nv, basis, sums);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -668,33 +688,18 @@ cudaError_t launch_step(int storage, int um, int nv, const void* src, void* dst,
     return step_storage(storage, um, nv, src, dst, a, st, basis, nullptr);
 }
 
-int64_t step_sum_blocks(int nx, int ny, int nv) {
-    return (int64_t)(((nx / nv) + 127) / 128) * (ny < 65535 ? ny : 65535);
-}
-
 int64_t step_sum_scratch(int nx, int ny, int nv) {
-    const int64_t nblk = step_sum_blocks(nx, ny, nv);
-    return 4 * nblk + 4 * ((nblk + kReduceThreads - 1) / kReduceThreads);
+    return 4 * (int64_t)(((nx / nv) + 127) / 128) * (ny < 65535 ? ny : 65535);
 }
 
 cudaError_t launch_step_conserved(int storage, int um, int nv, const void* src, void* dst,
                                   const StepArgs& a, cudaStream_t st, int basis, double rho_ref,
                                   double jx_ref, double jy_ref, double lambda,
-                                  double* partials, double* out) {
-    if (nv < 2 || !partials || !out) return cudaErrorInvalidValue;
-    int64_t nblk = 0;  // block slots the step writes (at most step_sum_blocks)
-    cudaError_t e = step_storage(storage, um, nv, src, dst, a, st, basis, partials, &nblk);
-    if (e != cudaSuccess) return e;
-    // the step's block partials, a fixed 256 per block of a middle level, then one block
-    const int64_t mid = (nblk + kReduceThreads - 1) / kReduceThreads;
-    double* mids = partials + 4 * nblk;
-    k_sum_partials<<<(unsigned)mid, kReduceThreads, 0, st>>>(partials, nblk, mids);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+                                  double* partials, unsigned* ticket, double* out) {
+    if (nv < 2 || !partials || !ticket || !out) return cudaErrorInvalidValue;
     const double n = (double)a.nx * (double)a.ny;
-    k_conserved_final<<<1, kReduceThreads, 0, st>>>(mids, (int)mid, rho_ref * n, jx_ref * n,
-                                                    jy_ref * n, lambda, out);
-    return cudaGetLastError();
+    const StepSums sums{partials, ticket, out, rho_ref * n, jx_ref * n, jy_ref * n, lambda};
+    return step_storage(storage, um, nv, src, dst, a, st, basis, &sums);
 }
 
 namespace {

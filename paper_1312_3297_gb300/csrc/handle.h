@@ -45,7 +45,7 @@ struct lbmrv_s {
     lbmrv::TilePlan tile;
     double* red = nullptr;   // reduction scratch: 8 * red_blocks partials + 8 results + ticket
     int red_blocks = 0;
-    double* fused = nullptr;  // partials of the step with fused sums, + 4 results (lazy)
+    double* fused = nullptr;  // step with fused sums: 6 results, ticket, partials (lazy)
     int64_t fused_doubles = 0;
     float* sin_x = nullptr;  // sin(2 pi x / nx) table of the analytic prescribed field
     // last lbmrv_forward_checkpointed: the adjoint must match it

@@ -80,13 +80,13 @@ cudaError_t launch_tile16(int storage, int um, int basis, int nv, const void* sr
                           cudaStream_t st);
 
 // The same step (nv >= 2) with the FP64 conserved sums of dst fused in, written to out[4]
-// as launch_conserved does; partials: step_sum_scratch(nx, ny, nv) doubles of scratch.
-int64_t step_sum_blocks(int nx, int ny, int nv);
+// as launch_conserved does; partials: step_sum_scratch(nx, ny, nv) doubles of scratch; ticket: a
+// device word that is 0 between calls.
 int64_t step_sum_scratch(int nx, int ny, int nv);
 cudaError_t launch_step_conserved(int storage, int um, int nv, const void* src, void* dst,
                                   const StepArgs& a, cudaStream_t st, int basis, double rho_ref,
                                   double jx_ref, double jy_ref, double lambda,
-                                  double* partials, double* out);
+                                  double* partials, unsigned* ticket, double* out);
 
 // Initial fields: density (or null: 1) and velocity components, n floats each.
 struct Fields {

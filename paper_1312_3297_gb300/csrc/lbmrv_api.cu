@@ -549,7 +549,7 @@ int lbmrv_step_conserved(lbmrv_t h, int64_t n, double out_host[5]) {
         ? step_sum_scratch((int)h->nx, (int)h->ny, nv)
         : step3_sum_scratch(h->storage, nv, make_args3(h, h->t + 1));
     if (scratch < 0) return cuda_fail(h, cudaGetLastError(), "lbmrv_step_conserved");
-    const int64_t need = scratch + 8;  // + the results
+    const int64_t need = 8 + scratch;  // results and ticket, then the blocks' partials
     if (need > h->fused_doubles) {
         cudaError_t e = cudaStreamSynchronize(h->stream);  // the old scratch may be in use
         if (e == cudaSuccess) e = cudaFree(h->fused);
@@ -557,25 +557,29 @@ int lbmrv_step_conserved(lbmrv_t h, int64_t n, double out_host[5]) {
         h->fused_doubles = 0;
         if (e == cudaSuccess)
             e = cudaMalloc(reinterpret_cast<void**>(&h->fused), sizeof(double) * need);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(h->fused, 0, 8 * sizeof(double), h->stream);
         if (e != cudaSuccess) {
             cudaGetLastError();
+            cudaFree(h->fused);
             h->fused = nullptr;
             return fail(h, LBMRV_E_NOMEM, "lbmrv_step_conserved: scratch of %lld doubles: %s",
                         (long long)need, cudaGetErrorString(e));
         }
         h->fused_doubles = need;
     }
-    double* res = h->fused + scratch;
+    double *res = h->fused, *part = h->fused + 8;
     cudaError_t e;
     if (h->dim == 2)
         e = launch_step_conserved(h->storage, kernel_mode(h), nv, h->f[h->cur], h->f[1 - h->cur],
                                   make_args(h, h->t + 1), h->stream, h->basis, h->rho_ref,
                                   h->rho_ref * h->u_ref[0] / h->lambda,
-                                  h->rho_ref * h->u_ref[1] / h->lambda, h->lambda, h->fused, res);
+                                  h->rho_ref * h->u_ref[1] / h->lambda, h->lambda, part,
+                                  reinterpret_cast<unsigned*>(res + 6), res);
     else
         e = launch_step3_conserved(h->storage, kernel_mode(h), nv, h->f[h->cur],
                                    h->f[1 - h->cur], make_args3(h, h->t + 1), h->stream,
-                                   h->lambda, h->fused, scratch, res);
+                                   h->lambda, part, scratch, res);
     if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step_conserved");
     h->cur = 1 - h->cur;
     h->t += 1;
