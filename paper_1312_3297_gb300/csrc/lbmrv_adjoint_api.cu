@@ -138,7 +138,6 @@ int lbmrv_adjoint(lbmrv_t h, int64_t n, int64_t seg, void* ws_dev, size_t ws_byt
     const int nv = choose_width(h, ws_dev, ws_dev);
     const int anv = adjoint_nv(h);
     double* acc = reinterpret_cast<double*>(at(ws_dev, L.off_acc));
-    double* res = acc + 8 * L.nblk;
     float* mu[2] = {reinterpret_cast<float*>(at(ws_dev, L.off_mu)),
                     reinterpret_cast<float*>(at(ws_dev, L.off_mu + L.mu))};
     cudaError_t e = cudaMemsetAsync(acc, 0, (size_t)L.nblk * 8 * sizeof(double), h->stream);
@@ -177,11 +176,9 @@ int lbmrv_adjoint(lbmrv_t h, int64_t n, int64_t seg, void* ws_dev, size_t ws_byt
         }
     }
     if (e == cudaSuccess) e = launch_gather(a, dL_dS0_dev, (int)h->nx, (int)h->ny, h->stream);
-    if (e == cudaSuccess) e = launch_acc_final(acc, L.nblk, res, h->stream);
+    if (e == cudaSuccess) e = launch_acc_final(acc, L.nblk, result_slot(h), h->stream);
     double out[8] = {0};
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out, res, sizeof(out), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) e = read_results(h, out, 8);
     if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_adjoint");
     if (dL_ds_host) {
         dL_ds_host[0] = dL_ds_host[1] = dL_ds_host[2] = 0.0;
@@ -228,13 +225,10 @@ int lbmrv_adjoint_acc_sum(lbmrv_t h, const double* acc_dev, double* dL_ds_host,
     if (h->lattice != LBMRV_D2Q9)
         return fail(h, LBMRV_E_UNSUPPORTED, "lbmrv_adjoint_acc_sum: needs a D2Q9 handle");
     DeviceGuard g(h->device);
-    double* res = h->red + 8 * (size_t)h->red_blocks;
     double out[8] = {0};
-    cudaError_t e = launch_acc_final(acc_dev, lbmrv_adjoint_acc_doubles(h) / 8 - 1, res,
-                                     h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out, res, sizeof(out), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    cudaError_t e = launch_acc_final(acc_dev, lbmrv_adjoint_acc_doubles(h) / 8 - 1,
+                                     result_slot(h), h->stream);
+    if (e == cudaSuccess) e = read_results(h, out, 8);
     if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_adjoint_acc_sum");
     if (dL_ds_host) {
         dL_ds_host[0] = dL_ds_host[1] = dL_ds_host[2] = 0.0;
@@ -259,7 +253,7 @@ int lbmrv_kinetic_energy(lbmrv_t h, double* ke_host, float* dL_dS_dev) {
     if (h->lattice != LBMRV_D2Q9)
         return fail(h, LBMRV_E_UNSUPPORTED, "lbmrv_kinetic_energy: needs a D2Q9 handle");
     DeviceGuard g(h->device);
-    double* res = h->red + 8 * (size_t)h->red_blocks;
+    double* const res = result_slot(h);
     cudaError_t e = cudaSuccess;
     if (h->slab && dL_dS_dev)  // the halo layers are not part of the loss
         e = cudaMemsetAsync(dL_dS_dev, 0, sizeof(float) * 9 * (size_t)h->n, h->stream);
@@ -270,9 +264,7 @@ int lbmrv_kinetic_energy(lbmrv_t h, double* ke_host, float* dL_dS_dev) {
                                   dL_dS_dev ? dL_dS_dev + o : nullptr, owned_count(h), h->n,
                                   store_ref(h), (float)h->lambda, h->red, h->red_blocks, res,
                                   h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ke_host, res, sizeof(double), cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) e = read_results(h, ke_host, 1);
     if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_kinetic_energy");
     return LBMRV_OK;
 }

@@ -54,15 +54,11 @@ void warn_rates(lbmrv_t h, int lattice, const double* s, const char* who) {
 }  // namespace
 
 cudaError_t flow_sums(const lbmrv_s* h, const Fields& f, int64_t n, double sums[4]) {
-    double* res = h->red + 8 * (size_t)h->red_blocks;
+    double* const res = result_slot(h);
+    unsigned* const ticket = reinterpret_cast<unsigned*>(h->sin_x + h->nx);
     for (int c = 0; c < 4; ++c) sums[c] = 0.0;
-    auto read = [&](cudaError_t e) {
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(sums, res, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
-        return e == cudaSuccess ? cudaStreamSynchronize(h->stream) : e;
-    };
-    cudaError_t e = read(launch_mean_flow(f, n, h->dim, h->red, h->red_blocks,
-                                          reinterpret_cast<unsigned*>(res + 8), res, h->stream));
+    cudaError_t e = launch_mean_flow(f, n, h->dim, h->red, h->red_blocks, ticket, res, h->stream);
+    if (e == cudaSuccess) e = read_results(h, sums, 4);
     if (e != cudaSuccess) return e;
     // densities far from 1, or momenta beyond FP32: the FP64 kernel
     const double mean = sums[0] / (double)n;
@@ -70,7 +66,8 @@ cudaError_t flow_sums(const lbmrv_s* h, const Fields& f, int64_t n, double sums[
                        std::isfinite(sums[2]) && std::isfinite(sums[3]) && mean > 1e-6 &&
                        mean < 1e6;
     if (usual) return cudaSuccess;
-    return read(launch_mean_flow_fp64(f, n, h->dim, h->red, h->red_blocks, res, h->stream));
+    e = launch_mean_flow_fp64(f, n, h->dim, h->red, h->red_blocks, res, h->stream);
+    return e == cudaSuccess ? read_results(h, sums, 4) : e;
 }
 
 namespace {
@@ -235,12 +232,11 @@ int lbmrv_create(lbmrv_t* out, int lattice, const int64_t dims[3], double lambda
         ok = cudaMalloc(&h->f[0], bytes) == cudaSuccess && cudaMalloc(&h->f[1], bytes) == cudaSuccess;
     }
     h->red_blocks = conserved_blocks(h->n);
-    ok = ok && cudaMalloc(&h->red, sizeof(double) * (8 * (size_t)h->red_blocks + 9)) == cudaSuccess;
-    // the reduction's ticket; done when the blocking copy below is
-    ok = ok && cudaMemset(h->red + 8 * (size_t)h->red_blocks + 8, 0, sizeof(double)) == cudaSuccess;
-    ok = ok && cudaMalloc(&h->sin_x, sizeof(float) * (size_t)h->nx) == cudaSuccess;
+    ok = ok && cudaMalloc(&h->red, sizeof(double) * (8 * (size_t)h->red_blocks + 8)) == cudaSuccess;
+    // the table, then the reductions' ticket (a zero word)
+    ok = ok && cudaMalloc(&h->sin_x, sizeof(float) * (size_t)(h->nx + 1)) == cudaSuccess;
     if (ok) {
-        std::vector<float> tab((size_t)h->nx);
+        std::vector<float> tab((size_t)h->nx + 1);
         for (int64_t x = 0; x < h->nx; ++x)
             tab[(size_t)x] = (float)std::sin(2.0 * M_PI * (double)x / (double)h->nx);
         ok = cudaMemcpy(h->sin_x, tab.data(), sizeof(float) * tab.size(),
@@ -258,6 +254,12 @@ int lbmrv_create(lbmrv_t* out, int lattice, const int64_t dims[3], double lambda
         return fail(nullptr, LBMRV_E_NOMEM, "lbmrv_create: device allocation of %zu bytes failed",
                     2 * bytes);
     }
+    void* host = nullptr;
+    if (cudaHostAlloc(&host, 8 * sizeof(double), cudaHostAllocMapped | cudaHostAllocPortable) ==
+        cudaSuccess)
+        h->host = static_cast<double*>(host);
+    else
+        cudaGetLastError();  // results are copied instead
     warn_rates(h, lattice, s, "lbmrv_create");
     warn_rates(nullptr, lattice, s, "lbmrv_create");
     *out = h;
@@ -275,6 +277,7 @@ int lbmrv_destroy(lbmrv_t h) {
     cudaFree(h->red);
     cudaFree(h->sin_x);
     cudaFree(h->fused);
+    if (h->host) cudaFreeHost(h->host);
     delete h;
     return LBMRV_OK;
 }
@@ -493,7 +496,7 @@ int lbmrv_conserved3(lbmrv_t h, double out_host[5]) {
     lbmrv::TraceRange trace("lbmrv_conserved");
     if (!h || !out_host) return fail(h, LBMRV_E_INVAL, "lbmrv_conserved3: NULL argument");
     DeviceGuard g(h->device);
-    double* res = h->red + 8 * (size_t)h->red_blocks;
+    double* const res = result_slot(h);
     cudaError_t e;
     double tmp[5] = {0, 0, 0, 0, 0};
     // a slab sums its interior layers only
@@ -506,9 +509,7 @@ int lbmrv_conserved3(lbmrv_t h, double out_host[5]) {
                              h->rho_ref * h->u_ref[0] / h->lambda,
                              h->rho_ref * h->u_ref[1] / h->lambda, h->lambda, h->red,
                              h->red_blocks, res, h->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(four, res, sizeof(four), cudaMemcpyDeviceToHost, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        if (e == cudaSuccess) e = read_results(h, four, 4);
         tmp[0] = four[0];
         tmp[1] = four[1];
         tmp[2] = four[2];
@@ -516,9 +517,7 @@ int lbmrv_conserved3(lbmrv_t h, double out_host[5]) {
     } else {
         e = launch_conserved3(h->storage, src, count, h->n, store_ref3(h), h->lambda, h->red,
                               h->red_blocks, res, h->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(tmp, res, sizeof(tmp), cudaMemcpyDeviceToHost, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        if (e == cudaSuccess) e = read_results(h, tmp, 5);
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_conserved");
     for (int k = 0; k < 5; ++k) out_host[k] = tmp[k];
@@ -549,7 +548,7 @@ int lbmrv_step_conserved(lbmrv_t h, int64_t n, double out_host[5]) {
         ? step_sum_scratch((int)h->nx, (int)h->ny, nv)
         : step3_sum_scratch(h->storage, nv, make_args3(h, h->t + 1));
     if (scratch < 0) return cuda_fail(h, cudaGetLastError(), "lbmrv_step_conserved");
-    const int64_t need = 8 + scratch;  // results and ticket, then the blocks' partials
+    const int64_t need = 8 + scratch;  // the ticket, then the blocks' partials
     if (need > h->fused_doubles) {
         cudaError_t e = cudaStreamSynchronize(h->stream);  // the old scratch may be in use
         if (e == cudaSuccess) e = cudaFree(h->fused);
@@ -568,14 +567,14 @@ int lbmrv_step_conserved(lbmrv_t h, int64_t n, double out_host[5]) {
         }
         h->fused_doubles = need;
     }
-    double *res = h->fused, *part = h->fused + 8;
+    double *const res = result_slot(h), *const part = h->fused + 8;
     cudaError_t e;
     if (h->dim == 2)
         e = launch_step_conserved(h->storage, kernel_mode(h), nv, h->f[h->cur], h->f[1 - h->cur],
                                   make_args(h, h->t + 1), h->stream, h->basis, h->rho_ref,
                                   h->rho_ref * h->u_ref[0] / h->lambda,
                                   h->rho_ref * h->u_ref[1] / h->lambda, h->lambda, part,
-                                  reinterpret_cast<unsigned*>(res + 6), res);
+                                  reinterpret_cast<unsigned*>(h->fused), res);
     else
         e = launch_step3_conserved(h->storage, kernel_mode(h), nv, h->f[h->cur],
                                    h->f[1 - h->cur], make_args3(h, h->t + 1), h->stream,
@@ -584,9 +583,7 @@ int lbmrv_step_conserved(lbmrv_t h, int64_t n, double out_host[5]) {
     h->cur = 1 - h->cur;
     h->t += 1;
     double five[5] = {0, 0, 0, 0, 0};
-    e = cudaMemcpyAsync(five, res, sizeof(double) * (h->dim == 2 ? 4 : 5),
-                        cudaMemcpyDeviceToHost, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    e = read_results(h, five, h->dim == 2 ? 4 : 5);
     if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step_conserved");
     if (h->dim == 2) {  // {rho, q_x, q_y, non-finite} -> the lbmrv_conserved3 layout
         five[4] = five[3];
