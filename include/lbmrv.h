@@ -132,7 +132,8 @@ LBMRV_API int64_t lbmrv_state_bytes(int lattice, const int64_t dims[3], int stor
  *            the caller and used as the A-B pair of the pull step; or both NULL, and
  *            the library allocates (and later frees) them.
  * The handle also allocates a small reduction buffer (under 64 KB), 64 bytes of mapped host
- * memory for results, and the nx-float table sin(2 pi x / nx) of the analytic prescribed field.
+ * memory for results (of 4 KB pages that the process's handles share; one page is kept for
+ * later handles), and the nx-float table sin(2 pi x / nx) of the analytic prescribed field.
  * Errors: LBMRV_E_INVAL, LBMRV_E_UNSUPPORTED, LBMRV_E_NOMEM, LBMRV_E_CUDA; *out is NULL. */
 LBMRV_API int lbmrv_create(lbmrv_t* out, int lattice, const int64_t dims[3], double lambda,
                  const double* s, int umode, int storage, double rho_ref, void* stream,

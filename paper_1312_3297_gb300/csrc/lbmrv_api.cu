@@ -5,6 +5,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -50,6 +51,71 @@ void warn_rates(lbmrv_t h, int lattice, const double* s, const char* who) {
                  who, k, s[k], (s[k] == 0.0 || s[k] == 2.0) ? "not damped" : "amplified");
             return;
         }
+}
+
+// Mapped host memory for the handles' results, 64 bytes each, cut from pages: pinning a page
+// and giving it back costs a create/destroy pair 60 - 200 us, a slot of a pinned one 1 us. A
+// page is given back when its last slot is, except one of 4 KB, which stays for the next handle.
+struct HostPage {
+    char* base;
+    uint64_t used;  // a bit per slot
+};
+constexpr int kSlotBytes = 64, kPageBytes = 64 * kSlotBytes, kMaxPages = 64;
+std::mutex g_pages_mutex;
+HostPage g_pages[kMaxPages];
+int g_page_count = 0;
+
+// Still pinned (a device reset frees the memory under the pool)?
+bool page_alive(const HostPage& p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p.base) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeHost;
+}
+
+// A slot, or null if no memory can be pinned or every page is full.
+double* acquire_host_slot() {
+    std::lock_guard<std::mutex> lock(g_pages_mutex);
+    for (int i = 0; i < g_page_count;) {
+        HostPage& p = g_pages[i];
+        if (!page_alive(p)) {
+            p = g_pages[--g_page_count];
+            continue;
+        }
+        for (int b = 0; b < 64; ++b)
+            if (!(p.used >> b & 1)) {
+                p.used |= (uint64_t)1 << b;
+                return reinterpret_cast<double*>(p.base + b * kSlotBytes);
+            }
+        ++i;
+    }
+    void* base = nullptr;
+    if (g_page_count == kMaxPages) return nullptr;
+    if (cudaHostAlloc(&base, kPageBytes, cudaHostAllocMapped | cudaHostAllocPortable) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    g_pages[g_page_count++] = {static_cast<char*>(base), 1};
+    return static_cast<double*>(base);
+}
+
+void release_host_slot(double* slot) {
+    if (!slot) return;
+    std::lock_guard<std::mutex> lock(g_pages_mutex);
+    char* const c = reinterpret_cast<char*>(slot);
+    for (int i = 0; i < g_page_count; ++i) {
+        HostPage& p = g_pages[i];
+        if (c < p.base || c >= p.base + kPageBytes) continue;
+        p.used &= ~((uint64_t)1 << (c - p.base) / kSlotBytes);
+        if (p.used == 0 && g_page_count > 1) {
+            cudaFreeHost(p.base);
+            p = g_pages[--g_page_count];
+        }
+        return;
+    }
 }
 }  // namespace
 
@@ -254,12 +320,7 @@ int lbmrv_create(lbmrv_t* out, int lattice, const int64_t dims[3], double lambda
         return fail(nullptr, LBMRV_E_NOMEM, "lbmrv_create: device allocation of %zu bytes failed",
                     2 * bytes);
     }
-    void* host = nullptr;
-    if (cudaHostAlloc(&host, 8 * sizeof(double), cudaHostAllocMapped | cudaHostAllocPortable) ==
-        cudaSuccess)
-        h->host = static_cast<double*>(host);
-    else
-        cudaGetLastError();  // results are copied instead
+    h->host = acquire_host_slot();  // null: results are copied instead
     warn_rates(h, lattice, s, "lbmrv_create");
     warn_rates(nullptr, lattice, s, "lbmrv_create");
     *out = h;
@@ -277,7 +338,7 @@ int lbmrv_destroy(lbmrv_t h) {
     cudaFree(h->red);
     cudaFree(h->sin_x);
     cudaFree(h->fused);
-    if (h->host) cudaFreeHost(h->host);
+    release_host_slot(h->host);
     delete h;
     return LBMRV_OK;
 }
