@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(256) k_step_scalar(const T* __restrict__ src,
 //
 // SUMS: also add up the conserved moments of the stored result (the values as rounded to
 // the storage type) in the block's slot part[4 * block] (sum g, sum c_x g, sum c_y g,
-// non-finite nodes), as k_conserved_partial does for a stored state; k_conserved_final then
+// non-finite nodes), as k_conserved_partial does for a stored state; the last block to finish
 // adds the slots in a fixed order. The launcher then sizes the grid to the blocks resident
 // at once, so each block walks many rows and its FP64 reduction runs once.
 // The paired cascaded relaxation (Geier's basis, 8-node packs) is held to five blocks per
