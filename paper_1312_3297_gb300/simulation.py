@@ -172,7 +172,8 @@ class D2Q9:
         u = torch.empty((self.DIM,) + self.shape, dtype=torch.float32, device=self.device)
         B.lbmrv_moments(self.h, rho, u)
         self._sync_out()
-        return (rho,) + u.unbind(0)
+        # separate views: unbind's outputs refuse in-place operations under autograd
+        return (rho,) + tuple(u[a] for a in range(self.DIM))
 
     def moments_host(self, rho_host=None, u_host=None):
         if rho_host is None:
