@@ -21,6 +21,12 @@ def mode_id(mode) -> int:
     return _MODES[mode] if isinstance(mode, str) else int(mode)
 
 
+def _in_memory(t: torch.Tensor) -> bool:
+    """Whether the tensor's memory holds its values: a lazily negated view (the imaginary part
+    of a conjugate) holds their negatives, a symbolic zero nothing."""
+    return not (t.is_neg() or t._is_zerotensor())
+
+
 def storage_id(storage) -> int:
     return _STORAGES[storage] if isinstance(storage, str) else int(storage)
 
@@ -146,7 +152,7 @@ class D2Q9:
             raise ValueError(f"expected {self.DIM} velocity components")
         rho = torch.as_tensor(rho, dtype=torch.float32, device=self.device).contiguous()
         u = [torch.as_tensor(c, dtype=torch.float32, device=self.device) for c in u_components]
-        if self._on_current_stream() and all(c.shape == u[0].shape for c in u):
+        if self._on_current_stream() and all(c.shape == u[0].shape and _in_memory(c) for c in u):
             u = [c.contiguous() for c in u]
             B.lbmrv_init_equilibrium_fields(self.h, rho, *u)
         else:  # read on another stream: a copy that the caller's tensors do not share

@@ -27,3 +27,25 @@ def test_a_field_can_be_changed_in_place_under_autograd(monkeypatch, k):
     field += p
     (3.0 * field).sum().backward()
     assert torch.equal(p.grad, torch.full((3, 4), 3.0))
+
+
+@pytest.mark.parametrize("kind", ["plain", "negated", "zero", "strided"])
+def test_init_reads_the_values_of_lazy_views(monkeypatch, kind):
+    """The library reads a field's memory: a view whose values are not what its memory holds
+    has to be written out first."""
+    got = []
+
+    def read(h, rho, *u):
+        assert all(c.is_contiguous() and not c.is_neg() for c in u)
+        got.append([c.reshape(-1).numpy().copy() for c in u])
+
+    sim = _wrapper(monkeypatch, lbmrv_init_equilibrium_fields=read,
+                   lbmrv_init_equilibrium=lambda h, rho, u: read(h, rho, *u))
+    base = torch.arange(12.0).reshape(3, 4)
+    field = {"plain": base, "negated": torch._neg_view(base),
+             "zero": torch._efficientzerotensor((3, 4)),
+             "strided": torch.arange(24.0).reshape(3, 8)[:, ::2]}[kind]
+    want = {"plain": base, "negated": -base, "zero": 0 * base,
+            "strided": 2 * base}[kind].reshape(-1).tolist()
+    sim.init_equilibrium(torch.ones(3, 4), field, base)
+    assert got[0][0].tolist() == want and got[0][1].tolist() == base.reshape(-1).tolist()
