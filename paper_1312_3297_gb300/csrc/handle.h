@@ -39,11 +39,8 @@ struct lbmrv_s {
     int64_t t = 0;
     const float* ut0 = nullptr;
     double amp = 0.0, period = 0.0;
-    // how lbmrv_step takes plan_n steps in mode plan_um (D2Q9, automatic kernel variant)
-    int64_t plan_n = 0;
-    int plan_um = -1;
-    bool march = false;
-    lbmrv::TilePlan tile;
+    // arrays of the tile kernel found so far: without, with a stored relative-velocity field
+    lbmrv::TileTable tiles[2];
     double* red = nullptr;   // reduction scratch: 8 * red_blocks partials + 8 results
     int red_blocks = 0;
     double* host = nullptr;  // 8 results that kernels write and the host reads (mapped memory)

@@ -54,7 +54,7 @@ cudaError_t launch_march(int storage, int um, const void* src, void* dst, const 
 // p.steps steps src -> dst in one launch on shared-memory tiles (d2q9_tile.cuh): arrays of p.rx
 // x p.ry nodes, blocks of p.warps warps. The bits of that many launch_step calls at pack width nv.
 constexpr int kTileMaxSteps = 12;
-constexpr int kTileMinSteps = 5;  // of a call: fewer are not worth planning (about 10 us, once)
+constexpr int kTileMinSteps = 5;  // of a call: fewer steps are left to the other forms
 constexpr int kTileMaxSmem = 224 * 1024;
 constexpr int kTileWarps = 24;  // most per block and per SM
 struct TileAmps {
@@ -67,11 +67,19 @@ struct TilePlan {
     int64_t launches = 0;  // for the n steps planned: `launches` passes of at most `steps`
     double us = 0.0;       // modelled time of the n steps
 };
+// The fastest array for a launch of s steps, found when it is first asked for. It depends on the
+// lattice only, so a handle searches once per s, whatever step counts it is called with. us: the
+// modelled time of that launch or, with steps = 1, a time that no array undercuts.
+struct TileTable {
+    TilePlan best[kTileMaxSteps + 1];
+};
 inline int64_t tile_bytes(int rx, int ry, int elem, int um) {
     return 9LL * rx * (ry + 3) * elem +
            (um == UM_FIELD ? 8LL * rx * (ry + 1) : um == UM_ANALYTIC ? 4LL * (ry + 1) : 0);
 }
-TilePlan tile_plan(int storage, int um, int nv, int nx, int ny, int64_t n);
+// Plan of n steps; steps = 1 unless it takes less than `least` microseconds.
+TilePlan tile_plan(TileTable& table, int storage, int um, int nv, int nx, int ny, int64_t n,
+                   double least);
 cudaError_t launch_tile(int storage, int um, int basis, int nv, const void* src, void* dst,
                         const StepArgs& a, const TileAmps& amps, const TilePlan& p,
                         cudaStream_t st);

@@ -416,7 +416,6 @@ int lbmrv_set_utilde(lbmrv_t h, const float* ut0_dev, double amplitude, double p
     if (h->lattice == LBMRV_D3Q19 && h->umode == LBMRV_UT_PRESCRIBED && !ut0_dev)
         return fail(h, LBMRV_E_UNSUPPORTED, "lbmrv_set_utilde: D3Q19 needs a u~0 field");
     h->ut0 = ut0_dev;
-    h->plan_n = 0;  // the choice of a step's form depends on the field's alignment
     h->amp = amplitude;
     h->period = period;
     return LBMRV_OK;
@@ -460,19 +459,25 @@ int lbmrv_init_equilibrium_host(lbmrv_t h, const float* rho_host, const float* u
                             "lbmrv_init_equilibrium_host");
 }
 
-// Which form of the D2Q9 step takes n steps in least time; kept for the next call of as many.
-static void plan_steps(lbmrv_t h, int nv, int um, int64_t n) {
-    if (h->plan_n == n && h->plan_um == um) return;
+// Which form of the D2Q9 step takes n >= kMarchSteps steps in least time.
+struct StepPlan {
+    bool march = false;
+    TilePlan tile;
+};
+static StepPlan plan_steps(lbmrv_t h, int nv, int um, int64_t n) {
     const int nx = (int)h->nx, ny = (int)h->ny;
     const double march = march_step_us(h->storage, um, h->basis, nx, ny, h->f[0], h->f[1], h->ut0);
     const double single = single_step_us(h->storage, um, nv, nx, ny);
-    h->tile = TilePlan();
-    h->tile.us = n * single;
-    if (n >= kTileMinSteps) h->tile = tile_plan(h->storage, um, nv, nx, ny, n);
+    StepPlan p;
+    p.tile.us = n * single;
+    if (n >= kTileMinSteps) {  // only where clearly less than single steps
+        const TilePlan t = tile_plan(h->tiles[um == UM_FIELD], h->storage, um, nv, nx, ny, n,
+                                     0.93 * n * single);
+        if (t.steps > 1) p.tile = t;
+    }
     const int64_t rest = n % kMarchSteps;
-    h->march = (n - rest) * march + rest * single < 0.95 * h->tile.us;
-    h->plan_n = n;
-    h->plan_um = um;
+    p.march = (n - rest) * march + rest * single < 0.95 * p.tile.us;
+    return p;
 }
 
 int lbmrv_step(lbmrv_t h, int64_t n) {
@@ -486,10 +491,10 @@ int lbmrv_step(lbmrv_t h, int64_t n) {
     int64_t k = 0;
     if (n >= kMarchSteps && h->dim == 2 && h->width == 0 && !h->slab) {
         const int um = kernel_mode(h);
-        plan_steps(h, nv, um, n);
+        const StepPlan plan = plan_steps(h, nv, um, n);
         // passes of kMarchSteps steps; an odd number of steps per pass leaves every state in
         // the buffer that as many single steps would leave it in
-        for (; h->march && n - k >= kMarchSteps; k += kMarchSteps) {
+        for (; plan.march && n - k >= kMarchSteps; k += kMarchSteps) {
             MarchAmps amps;
             for (int l = 0; l < kMarchSteps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);
             cudaError_t e = launch_march(h->storage, um, h->f[h->cur], h->f[1 - h->cur],
@@ -499,8 +504,8 @@ int lbmrv_step(lbmrv_t h, int64_t n) {
             h->t += kMarchSteps;
         }
         // passes over shared-memory tiles, of equal lengths to within one
-        TilePlan p = h->tile;
-        for (int64_t m = h->march ? 0 : p.launches; m > 0; --m) {
+        TilePlan p = plan.tile;
+        for (int64_t m = plan.march ? 0 : p.launches; m > 0; --m) {
             p.steps = (int)((n - k + m - 1) / m);
             TileAmps amps;
             for (int l = 0; l < p.steps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);
