@@ -1,9 +1,10 @@
 """Differentiable rollout of the relative-velocity scheme for PyTorch.
 
 ``Rollout.apply(u0, s_nu, amp, sim, n, seg, rho0)`` sets the state of ``sim`` to the
-equilibrium of (rho0, u0), advances n steps with checkpoints every ``seg`` steps (None or 0:
-as few steps between them as a sixteenth of the device's memory allows, see
-``checkpoint_interval``; the gradient does not depend on it, bit for bit), and returns the final density and velocity fields. Its backward pass runs the hand-written
+equilibrium of (rho0, u0), advances n steps with checkpoints every ``seg`` steps, and returns
+the final density and velocity fields. With ``seg`` None or 0 the checkpoints are as dense as a
+sixteenth of the free memory allows, see ``default_workspace``; the gradient does not depend on
+the interval, bit for bit. The backward pass runs the hand-written
 discrete adjoint of the library (moments adjoint, reverse sweep, equilibrium adjoint),
 giving gradients with respect to the initial velocity field, the shear rate s_nu (the
 shared rate of p_xx and p_xy) and the amplitude of a prescribed relative velocity.
@@ -12,25 +13,67 @@ All arithmetic runs in the CUDA library; this module only moves tensors.
 from __future__ import annotations
 
 import math
+import threading
+import weakref
 
 import torch
 
 
-# Share of the device's memory that a rollout's checkpoints may take by default.
+# Share of a device's memory that checkpoints may take without being asked for.
 CHECKPOINT_SHARE = 1 / 16
 
+# Bytes that the workspaces alive on each device hold beyond those of sqrt(n) checkpoints.
+_extra: dict = {}
+_extra_lock = threading.RLock()  # a workspace may be collected while its own thread holds it
 
-def checkpoint_interval(sim, n: int) -> int:
-    """The shortest checkpoint interval whose workspace stays within CHECKPOINT_SHARE of the
-    device's memory, at most sqrt(n) (the least memory). Every step within an interval is
-    recomputed before it is reversed, a quarter of a gradient's time with sqrt(n): 200 steps at
-    1024^2 take 7.8 ms with 15 steps between checkpoints (1.2 GB) and 6.1 ms with none (7.6 GB)."""
+
+def checkpoint_interval(sim, n: int, budget: float | None = None) -> int:
+    """The shortest checkpoint interval whose workspace stays within `budget` bytes (default:
+    CHECKPOINT_SHARE of the device's memory), at most sqrt(n), which needs the least. Every step
+    within an interval is recomputed before it is reversed, a quarter of a gradient's time with
+    sqrt(n): 200 steps at 1024^2 take 7.8 ms with 15 steps between checkpoints (1.2 GB) and
+    6.1 ms with none (7.6 GB)."""
     longest = max(1, math.ceil(math.sqrt(n)))
-    budget = CHECKPOINT_SHARE * torch.cuda.get_device_properties(sim.device).total_memory
+    if budget is None:
+        budget = CHECKPOINT_SHARE * torch.cuda.get_device_properties(sim.device).total_memory
     for seg in range(1, longest):
         if sim.adjoint_workspace_bytes(n, seg) <= budget:
             return seg
     return longest
+
+
+def _give_back(device, nbytes: int):
+    with _extra_lock:
+        _extra[device] -= nbytes
+
+
+def default_workspace(sim, n: int):
+    """Checkpoint interval and workspace of a rollout that names no interval. What it holds
+    beyond sqrt(n) checkpoints, together with what all others alive on the device hold beyond
+    theirs, stays within CHECKPOINT_SHARE of the memory that the driver would have free with
+    sqrt(n) checkpoints only: a program that keeps many rollouts alive, or that leaves little memory free, gets
+    sqrt(n) checkpoints, as it does where the allocation fails."""
+    longest = max(1, math.ceil(math.sqrt(n)))
+    least = sim.adjoint_workspace_bytes(n, longest)
+    device = str(sim.device)
+    with _extra_lock:
+        held = _extra.setdefault(device, 0)
+        room = 0.0
+        if longest > 1:
+            spare = torch.cuda.mem_get_info(sim.device)[0] + held - least
+            room = CHECKPOINT_SHARE * max(0, spare) - held
+        seg = checkpoint_interval(sim, n, least + room)
+        more = max(0, sim.adjoint_workspace_bytes(n, seg) - least)
+        _extra[device] += more
+    try:
+        ws = sim.adjoint_workspace(n, seg)
+    except BaseException as e:
+        _give_back(device, more)
+        if more == 0 or not isinstance(e, torch.cuda.OutOfMemoryError):
+            raise
+        return longest, sim.adjoint_workspace(n, longest)
+    weakref.finalize(ws, _give_back, device, more)
+    return seg, ws
 
 
 class Rollout(torch.autograd.Function):
@@ -48,12 +91,7 @@ class Rollout(torch.autograd.Function):
             seg = int(seg)
             ws = sim.adjoint_workspace(n, seg)
         else:
-            seg = checkpoint_interval(sim, n)
-            try:
-                ws = sim.adjoint_workspace(n, seg)
-            except torch.cuda.OutOfMemoryError:  # others hold the memory: the least that serves
-                seg = max(1, math.ceil(math.sqrt(n)))
-                ws = sim.adjoint_workspace(n, seg)
+            seg, ws = default_workspace(sim, n)
         sim.forward_checkpointed(n, seg, ws)
         rho, ux, uy = sim.moments()
         ctx.sim, ctx.n, ctx.seg, ctx.ws = sim, n, seg, ws
