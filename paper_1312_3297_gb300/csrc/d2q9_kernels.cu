@@ -108,10 +108,16 @@ __device__ __forceinline__ bool last_block(unsigned* ticket, unsigned nblk) {
 // reference state's added.
 struct StepSums {
     double* part;
-    unsigned* ticket;  // 0 between launches
+    unsigned* ticket;  // 0 between launches; null: the slots are left to k_sum_slots
     double* out;
     double rho_n, jx_n, jy_n, lambda;
 };
+
+// Most slots that the step's last block adds. A slot takes it 3.6 ns; the two launches that add
+// them otherwise take 11 us whatever their number. Only rows of more than 4096 blocks of packs
+// have more (FP32 4,194,304 x 1, 8192 slots: 131 us a step with the last block, 120 without;
+// 33,554,432 x 1 893 and 741).
+constexpr int kLastBlockSlots = 4096;
 
 template <typename T, int UM, int BASIS>
 __global__ void __launch_bounds__(256) k_step_scalar(const T* __restrict__ src,
@@ -302,7 +308,7 @@ __global__ void __launch_bounds__(128, (step_vec_min_blocks<T, BASIS, NV, UM, SU
         // The last block to finish adds the slots, in a fixed order, and leaves *ticket at 0
         // again (two more launches took 11 us for this).
         const int nblk = gridDim.x * gridDim.y;
-        if (!last_block(o.ticket, nblk)) return;
+        if (!o.ticket || !last_block(o.ticket, nblk)) return;
 #pragma unroll
         for (int c = 0; c < 4; ++c) v[c] = 0.0;
         for (int b = threadIdx.x; b < nblk; b += 128) {
@@ -477,6 +483,18 @@ __global__ void __launch_bounds__(kReduceThreads) k_conserved_final(const double
     }
 }
 
+// Block b adds slots [256 b, 256 b + 256) of 4 doubles each into out[4 b].
+__global__ void __launch_bounds__(kReduceThreads) k_sum_slots(const double* __restrict__ part,
+                                                              int nblk, double* __restrict__ out) {
+    const int i = blockIdx.x * kReduceThreads + threadIdx.x;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    if (i < nblk) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = part[4 * (int64_t)i + c];
+    }
+    block_sum4<kReduceThreads>(v, out + 4 * (int64_t)blockIdx.x);
+}
+
 // Sum of FP32 terms kept in three FP32 parts whose sum is exact to about 2^-70 of it: the
 // rounding errors of the additions (and of the products) are carried along, by Knuth's two-sum
 // and Dekker's product with a fused multiply-add. Written with the single-operation
@@ -582,11 +600,23 @@ cudaError_t launch_vec(const T* s, T* d, const StepArgs& a, cudaStream_t st,
     auto kernel = k_step_vec<T, NV, UM, BASIS, true>;
     static std::atomic<int> resident[kMaxDevicesOcc];
     int full = 0;
-    const cudaError_t e = resident_blocks(kernel, resident, 128, 0, 32, &full);
+    cudaError_t e = resident_blocks(kernel, resident, 128, 0, 32, &full);
     if (e != cudaSuccess) return e;
     const int per_x = full / gx;
     const int gy = per_x < 1 ? 1 : (per_x < rows ? per_x : rows);
-    return launch_pdl(kernel, dim3(gx, gy), dim3(128), st, s, d, a, *sums);
+    const int nblk = gx * gy;
+    StepSums o = *sums;
+    if (nblk > kLastBlockSlots) o.ticket = nullptr;
+    e = launch_pdl(kernel, dim3(gx, gy), dim3(128), st, s, d, a, o);
+    if (e != cudaSuccess || o.ticket) return e;
+    const int mid = (nblk + kReduceThreads - 1) / kReduceThreads;
+    double* const mids = o.part + 4 * (int64_t)nblk;
+    k_sum_slots<<<mid, kReduceThreads, 0, st>>>(o.part, nblk, mids);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_conserved_final<<<1, kReduceThreads, 0, st>>>(mids, mid, o.rho_n, o.jx_n, o.jy_n, o.lambda,
+                                                    o.out);
+    return cudaGetLastError();
 }
 
 template <typename T, int UM, int BASIS>
@@ -688,8 +718,17 @@ cudaError_t launch_step(int storage, int um, int nv, const void* src, void* dst,
     return step_storage(storage, um, nv, src, dst, a, st, basis, nullptr);
 }
 
+// A single row of more blocks than the last block adds: every block would reduce for one pack
+// per thread, and the separate pass is cheaper.
+bool step_fuses_sums(int nx, int ny, int nv) {
+    return nv >= 2 && (ny > 1 || nx / nv <= 128 * kLastBlockSlots);
+}
+
 int64_t step_sum_scratch(int nx, int ny, int nv) {
-    return 4 * (int64_t)(((nx / nv) + 127) / 128) * (ny < 65535 ? ny : 65535);
+    // the blocks' slots, at most; with more than the last block adds, one per 256 of them too
+    const int64_t nblk = (int64_t)(((nx / nv) + 127) / 128) * (ny < 65535 ? ny : 65535);
+    return 4 * nblk + (nblk > kLastBlockSlots ? 4 * ((nblk + kReduceThreads - 1) / kReduceThreads)
+                                              : 0);
 }
 
 cudaError_t launch_step_conserved(int storage, int um, int nv, const void* src, void* dst,

@@ -89,7 +89,9 @@ cudaError_t launch_tile16(int storage, int um, int basis, int nv, const void* sr
 
 // The same step (nv >= 2) with the FP64 conserved sums of dst fused in, written to out[4]
 // as launch_conserved does; partials: step_sum_scratch(nx, ny, nv) doubles of scratch; ticket: a
-// device word that is 0 between calls.
+// device word that is 0 between calls. step_fuses_sums: whether that beats the step followed by
+// launch_conserved.
+bool step_fuses_sums(int nx, int ny, int nv);
 int64_t step_sum_scratch(int nx, int ny, int nv);
 cudaError_t launch_step_conserved(int storage, int um, int nv, const void* src, void* dst,
                                   const StepArgs& a, cudaStream_t st, int basis, double rho_ref,

@@ -601,7 +601,7 @@ int lbmrv_step_conserved(lbmrv_t h, int64_t n, double out_host[5]) {
     if (rc != LBMRV_OK) return rc;
     DeviceGuard g(h->device);
     const int nv = choose_width(h, h->f[0], h->f[1]);
-    const bool fused = !h->slab && (h->dim == 2 ? nv >= 2
+    const bool fused = !h->slab && (h->dim == 2 ? step_fuses_sums((int)h->nx, (int)h->ny, nv)
                                                 : step3_fuses_sums(h->storage, nv, (int)h->ny,
                                                                    (int)h->nz));
     if (!fused) {  // no fused form for this kernel: the step, then the sums' own pass

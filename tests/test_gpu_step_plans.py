@@ -50,3 +50,28 @@ def test_changing_step_counts_are_not_planned_again():
     assert _host_us_per_call(torch, sim, [new, five]) <= 2.0 * (
         _host_us_per_call(torch, sim, [five]) + _host_us_per_call(torch, sim, [new])) / 2
     sim.close()
+
+
+@pytest.mark.parametrize("storage,lanes", [("fp32", 512), ("fp16", 1024)])
+@pytest.mark.parametrize("blocks,ny", [(4096, 1), (4097, 1), (4096, 2), (4097, 2), (66000, 2)])
+def test_fused_sums_of_very_wide_rows(storage, lanes, blocks, ny):
+    """Rows of as many blocks as the step's last block adds, one more, and of more than 256
+    middle sums: the separate pass's sums, the same in every run."""
+    import numpy as np
+    import torch
+
+    from paper_1312_3297_gb300 import D2Q9
+
+    nx = (blocks - 1) * lanes + 8  # the last block holds one or two packs
+    sim = D2Q9(nx, ny, S, storage=storage)
+    gen = torch.Generator(device="cuda").manual_seed(blocks)
+    r = [torch.randn(ny, nx, generator=gen, device="cuda") for _ in range(3)]
+    runs = []
+    for _ in range(2):
+        sim.init_equilibrium(1.0 + 0.01 * r[0], 0.05 + 0.01 * r[1], 0.02 + 0.01 * r[2])
+        runs.append([sim.step_conserved(1) for _ in range(2)])
+    # the tolerance of the other fused sums: FP32 runs of 32 nodes, then FP64
+    np.testing.assert_allclose(runs[0][1][:4], sim.conserved3()[:4], rtol=1e-12,
+                               atol=1e-9 * nx * ny)
+    assert runs[0] == runs[1] and runs[0][1][4] == 0.0
+    sim.close()
