@@ -180,6 +180,25 @@ LBMRV_API int lbmrv_set_stream(lbmrv_t h, void* stream);
  * adjoint kernel. */
 LBMRV_API int lbmrv_set_kernel_width(lbmrv_t h, int nodes_per_thread);
 
+/* Form in which lbmrv_step takes the steps of one call (D2Q9): LBMRV_FORM_AUTO chooses by
+ * modelled time, the others force one launch per step, three steps per pass over memory
+ * (march; rows of whole 4-node packs in aligned buffers) or several per launch on
+ * shared-memory tiles. Steps that do not fill a forced form, a nonzero kernel width and slab
+ * handles take single steps. All forms give the same states bit for bit; this exists for
+ * testing and tuning. Errors: LBMRV_E_INVAL; LBMRV_E_UNSUPPORTED (the lattice has no such
+ * form); the form is then unchanged. */
+#define LBMRV_FORM_AUTO 0
+#define LBMRV_FORM_SINGLE 1
+#define LBMRV_FORM_MARCH 2
+#define LBMRV_FORM_TILE 3
+LBMRV_API int lbmrv_set_step_form(lbmrv_t h, int form);
+
+/* How lbmrv_step(h, n) would take n >= 0 steps now: out[0] the form (LBMRV_FORM_*, single if
+ * every launch is one step), out[1] the number of kernel launches, out[2] the steps of the
+ * longest launch, out[3] the width in nodes of the tile form's arrays (else 0). Launches
+ * nothing. */
+LBMRV_API int lbmrv_step_plan(lbmrv_t h, int64_t n, int64_t out[4]);
+
 /* Prescribed relative velocity u~(x, t) = amplitude * u~0(x) * cos(2 pi t / period),
  * evaluated at the time index t of each relaxation; period <= 0 means no time factor.
  *   ut0_dev  device FP32 [d][n] (one plane per component), kept by reference; or, for

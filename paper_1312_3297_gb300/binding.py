@@ -30,6 +30,10 @@ LBMRV_UT_PRESCRIBED = 2
 LBMRV_FP32 = 0
 LBMRV_FP16 = 1
 LBMRV_BF16 = 2
+LBMRV_FORM_AUTO = 0
+LBMRV_FORM_SINGLE = 1
+LBMRV_FORM_MARCH = 2
+LBMRV_FORM_TILE = 3
 
 _STATUS_NAMES = {
     LBMRV_E_INVAL: "LBMRV_E_INVAL", LBMRV_E_CUDA: "LBMRV_E_CUDA",
@@ -52,6 +56,8 @@ SIGNATURES = [
     ("lbmrv_last_error", ctypes.c_char_p, [_VP]),
     ("lbmrv_set_stream", _I, [_VP, _VP]),
     ("lbmrv_set_kernel_width", _I, [_VP, _I]),
+    ("lbmrv_set_step_form", _I, [_VP, _I]),
+    ("lbmrv_step_plan", _I, [_VP, _I64, ctypes.POINTER(_I64)]),
     ("lbmrv_set_utilde", _I, [_VP, _VP, _D, _D]),
     ("lbmrv_init_equilibrium", _I, [_VP, _VP, _VP]),
     ("lbmrv_init_equilibrium_fields", _I, [_VP, _VP, _VP, _VP, _VP]),
@@ -193,6 +199,17 @@ def lbmrv_set_stream(h, stream) -> None:
 
 def lbmrv_set_kernel_width(h, nodes_per_thread: int) -> None:
     _check(load().lbmrv_set_kernel_width(h, int(nodes_per_thread)), h)
+
+
+def lbmrv_set_step_form(h, form: int) -> None:
+    _check(load().lbmrv_set_step_form(h, int(form)), h)
+
+
+def lbmrv_step_plan(h, n: int) -> tuple:
+    """(form, launches, steps of the longest launch, tile width) of lbmrv_step(h, n)."""
+    out = (_I64 * 4)()
+    _check(load().lbmrv_step_plan(h, int(n), out), h)
+    return tuple(out)
 
 
 def lbmrv_set_utilde(h, ut0, amplitude: float, period: float) -> None:

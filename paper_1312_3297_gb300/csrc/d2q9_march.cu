@@ -383,10 +383,10 @@ double march_step_us(int storage, int um, int basis, int nx, int ny, const void*
     const int bytes = storage == kStoreF32 ? 16 : 8;
     if (nx % kNV != 0 || reinterpret_cast<uintptr_t>(a) % bytes != 0 ||
         reinterpret_cast<uintptr_t>(b) % bytes != 0)
-        return 1e30;
+        return kNoForm;
     if (um == UM_FIELD && (reinterpret_cast<uintptr_t>(ut0) % 16 != 0 ||
                            (storage != kStoreF32 && basis == 1 && nx % 8 != 0)))
-        return 1e30;
+        return kNoForm;
     // Measured on GB300: 0.235 nodes per ns and lane in use with every warp resident, 0.205
     // with half of them, 6 rows repeated in three per segment, a third of a launch.
     const int64_t warps = (int64_t)(um == UM_FIELD ? 12 : 16) * sm_count();

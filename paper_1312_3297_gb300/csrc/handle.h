@@ -41,6 +41,7 @@ struct lbmrv_s {
     double amp = 0.0, period = 0.0;
     // arrays of the tile kernel found so far: without, with a stored relative-velocity field
     lbmrv::TileTable tiles[2];
+    int form = 0;  // LBMRV_FORM_*
     double* red = nullptr;   // reduction scratch: 8 * red_blocks partials + 8 results
     int red_blocks = 0;
     double* host = nullptr;  // 8 results that kernels write and the host reads (mapped memory)

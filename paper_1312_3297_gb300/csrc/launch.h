@@ -36,8 +36,9 @@ cudaError_t launch_step(int storage, int um, int nv, const void* src, void* dst,
 int sm_count();
 
 // Modelled times of one step in microseconds, for the choice between the forms of the D2Q9
-// step: one launch per step at pack width nv; one of launch_march's three (1e30 where it does
+// step: one launch per step at pack width nv; one of launch_march's three (kNoForm where it does
 // not suit the lattice: row length, alignment; ut0 the stored field, or null).
+constexpr double kNoForm = 1e30;
 double single_step_us(int storage, int um, int nv, int nx, int ny);
 double march_step_us(int storage, int um, int basis, int nx, int ny, const void* a,
                      const void* b, const float* ut0);

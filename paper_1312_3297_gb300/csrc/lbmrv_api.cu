@@ -459,25 +459,70 @@ int lbmrv_init_equilibrium_host(lbmrv_t h, const float* rho_host, const float* u
                             "lbmrv_init_equilibrium_host");
 }
 
-// Which form of the D2Q9 step takes n >= kMarchSteps steps in least time.
+// How n steps are split into launches: `marches` passes of kMarchSteps steps, or tile.launches
+// passes over tiles, and single steps for the rest.
 struct StepPlan {
-    bool march = false;
+    int64_t marches = 0;
     TilePlan tile;
 };
-static StepPlan plan_steps(lbmrv_t h, int nv, int um, int64_t n) {
-    const int nx = (int)h->nx, ny = (int)h->ny;
-    const double march = march_step_us(h->storage, um, h->basis, nx, ny, h->f[0], h->f[1], h->ut0);
-    const double single = single_step_us(h->storage, um, nv, nx, ny);
+static StepPlan plan_steps(lbmrv_t h, int nv, int64_t n) {
     StepPlan p;
+    if (n < 2 || h->dim != 2 || h->width != 0 || h->slab || h->form == LBMRV_FORM_SINGLE) return p;
+    const int nx = (int)h->nx, ny = (int)h->ny, um = kernel_mode(h);
+    const int64_t rest = n % kMarchSteps;
+    const double march = march_step_us(h->storage, um, h->basis, nx, ny, h->f[0], h->f[1], h->ut0);
+    if (h->form == LBMRV_FORM_MARCH) {
+        if (march < kNoForm) p.marches = n / kMarchSteps;
+        return p;
+    }
+    if (h->form == LBMRV_FORM_TILE) {
+        TileTable table;  // the handle's own holds times below those of single steps only
+        p.tile = tile_plan(table, h->storage, um, nv, nx, ny, n, kNoForm);
+        return p;
+    }
+    if (n < kMarchSteps) return p;
+    // The form with the least modelled time.
+    const double single = single_step_us(h->storage, um, nv, nx, ny);
     p.tile.us = n * single;
     if (n >= kTileMinSteps) {  // only where clearly less than single steps
         const TilePlan t = tile_plan(h->tiles[um == UM_FIELD], h->storage, um, nv, nx, ny, n,
                                      0.93 * n * single);
         if (t.steps > 1) p.tile = t;
     }
-    const int64_t rest = n % kMarchSteps;
-    p.march = (n - rest) * march + rest * single < 0.95 * p.tile.us;
+    if ((n - rest) * march + rest * single < 0.95 * p.tile.us) {
+        p.marches = n / kMarchSteps;
+        p.tile = TilePlan();
+    }
     return p;
+}
+
+int lbmrv_set_step_form(lbmrv_t h, int form) {
+    if (!h) return fail(nullptr, LBMRV_E_INVAL, "lbmrv_set_step_form: NULL handle");
+    if (form < LBMRV_FORM_AUTO || form > LBMRV_FORM_TILE)
+        return fail(h, LBMRV_E_INVAL, "lbmrv_set_step_form: bad form %d", form);
+    if (form > LBMRV_FORM_SINGLE && h->dim != 2)
+        return fail(h, LBMRV_E_UNSUPPORTED, "lbmrv_set_step_form: needs a D2Q9 handle");
+    if (form == LBMRV_FORM_MARCH &&
+        march_step_us(h->storage, kernel_mode(h), h->basis, (int)h->nx, (int)h->ny, h->f[0],
+                      h->f[1], h->ut0) >= kNoForm)
+        return fail(h, LBMRV_E_UNSUPPORTED,
+                    "lbmrv_set_step_form: rows or buffers do not suit the marching form");
+    h->form = form;
+    return LBMRV_OK;
+}
+
+int lbmrv_step_plan(lbmrv_t h, int64_t n, int64_t out[4]) {
+    if (!h || !out) return fail(h, LBMRV_E_INVAL, "lbmrv_step_plan: NULL argument");
+    if (n < 0) return fail(h, LBMRV_E_INVAL, "lbmrv_step_plan: n < 0");
+    DeviceGuard g(h->device);
+    const StepPlan p = plan_steps(h, choose_width(h, h->f[0], h->f[1]), n);
+    out[0] = p.marches ? LBMRV_FORM_MARCH : p.tile.launches ? LBMRV_FORM_TILE : LBMRV_FORM_SINGLE;
+    out[1] = p.marches        ? p.marches + n - p.marches * kMarchSteps
+             : p.tile.launches ? p.tile.launches
+                               : n;
+    out[2] = p.marches ? kMarchSteps : p.tile.launches ? p.tile.steps : n > 0;
+    out[3] = p.tile.launches ? p.tile.rx : 0;
+    return LBMRV_OK;
 }
 
 int lbmrv_step(lbmrv_t h, int64_t n) {
@@ -487,36 +532,32 @@ int lbmrv_step(lbmrv_t h, int64_t n) {
     if (h->lattice == LBMRV_D3Q19 && h->umode == LBMRV_UT_PRESCRIBED && !h->ut0)
         return fail(h, LBMRV_E_INVAL, "lbmrv_step: D3Q19 prescribed mode needs a u~0 field");
     DeviceGuard g(h->device);
-    const int nv = choose_width(h, h->f[0], h->f[1]);
+    const int nv = choose_width(h, h->f[0], h->f[1]), um = kernel_mode(h);
+    StepPlan plan = plan_steps(h, nv, n);
     int64_t k = 0;
-    if (n >= kMarchSteps && h->dim == 2 && h->width == 0 && !h->slab) {
-        const int um = kernel_mode(h);
-        const StepPlan plan = plan_steps(h, nv, um, n);
-        // passes of kMarchSteps steps; an odd number of steps per pass leaves every state in
-        // the buffer that as many single steps would leave it in
-        for (; plan.march && n - k >= kMarchSteps; k += kMarchSteps) {
-            MarchAmps amps;
-            for (int l = 0; l < kMarchSteps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);
-            cudaError_t e = launch_march(h->storage, um, h->f[h->cur], h->f[1 - h->cur],
-                                         make_args(h, h->t + 1), amps, h->stream, h->basis);
-            if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step");
-            h->cur = 1 - h->cur;
-            h->t += kMarchSteps;
-        }
-        // passes over shared-memory tiles, of equal lengths to within one
-        TilePlan p = plan.tile;
-        for (int64_t m = plan.march ? 0 : p.launches; m > 0; --m) {
-            p.steps = (int)((n - k + m - 1) / m);
-            TileAmps amps;
-            for (int l = 0; l < p.steps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);
-            cudaError_t e = launch_tile(h->storage, um, h->basis, nv, h->f[h->cur],
-                                        h->f[1 - h->cur], make_args(h, h->t + 1), amps, p,
-                                        h->stream);
-            if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step");
-            h->cur = 1 - h->cur;
-            h->t += p.steps;
-            k += p.steps;
-        }
+    // passes of kMarchSteps steps; an odd number of steps per pass leaves every state in
+    // the buffer that as many single steps would leave it in
+    for (int64_t m = plan.marches; m > 0; --m, k += kMarchSteps) {
+        MarchAmps amps;
+        for (int l = 0; l < kMarchSteps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);
+        cudaError_t e = launch_march(h->storage, um, h->f[h->cur], h->f[1 - h->cur],
+                                     make_args(h, h->t + 1), amps, h->stream, h->basis);
+        if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step");
+        h->cur = 1 - h->cur;
+        h->t += kMarchSteps;
+    }
+    // passes over shared-memory tiles, of equal lengths to within one
+    for (int64_t m = plan.tile.launches; m > 0; --m) {
+        TilePlan& p = plan.tile;
+        p.steps = (int)((n - k + m - 1) / m);
+        TileAmps amps;
+        for (int l = 0; l < p.steps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);
+        cudaError_t e = launch_tile(h->storage, um, h->basis, nv, h->f[h->cur],
+                                    h->f[1 - h->cur], make_args(h, h->t + 1), amps, p, h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step");
+        h->cur = 1 - h->cur;
+        h->t += p.steps;
+        k += p.steps;
     }
     for (; k < n; ++k) {
         cudaError_t e = launch_handle_step(h, nv, h->f[h->cur], h->f[1 - h->cur], h->t + 1);

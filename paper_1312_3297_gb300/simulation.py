@@ -13,6 +13,7 @@ from . import binding as B
 _MODES = {"zero": B.LBMRV_UT_ZERO, "fluid": B.LBMRV_UT_FLUID,
           "prescribed": B.LBMRV_UT_PRESCRIBED}
 _STORAGES = {"fp32": B.LBMRV_FP32, "fp16": B.LBMRV_FP16, "bf16": B.LBMRV_BF16}
+_FORMS = ("auto", "single", "march", "tile")  # LBMRV_FORM_*
 STORAGE_DTYPES = {B.LBMRV_FP32: torch.float32, B.LBMRV_FP16: torch.float16,
                   B.LBMRV_BF16: torch.bfloat16}
 
@@ -130,6 +131,15 @@ class D2Q9:
 
     def set_kernel_width(self, nodes_per_thread: int):
         B.lbmrv_set_kernel_width(self.h, nodes_per_thread)
+
+    def set_step_form(self, form: str):
+        """Form of a call's steps: "auto", "single", "march" or "tile" (the same states)."""
+        B.lbmrv_set_step_form(self.h, _FORMS.index(form))
+
+    def step_plan(self, n: int) -> tuple:
+        """(form, kernel launches, steps of the longest launch, tile width) of ``step(n)``."""
+        form, *rest = B.lbmrv_step_plan(self.h, n)
+        return _FORMS[form], *rest
 
     def set_rates(self, s):
         B.lbmrv_set_rates(self.h, list(s))
