@@ -34,10 +34,12 @@ namespace {
 
 constexpr int kLevels = kMarchSteps;
 constexpr int kNV = 4;  // nodes per pack
-// Packs of a strip that are stored: each level loses one node at both ends of a strip, whose
-// neighbours belong to the next strips, so lanes 0 and 31 are recomputed there (kLevels <= kNV
-// + 1 keeps the loss within those lanes).
+// Packs of a strip that are stored: each level, the first too, leaves one wrong node more at
+// both ends of a strip, whose neighbours belong to the next strips, so lanes 0 and 31 are
+// recomputed there. The last level must still find a right node in them.
 constexpr int kUse = 30;
+static_assert(kLevels <= kNV, "wrong nodes would reach the lanes that are stored");
+static_assert(kLevels % 2 == 1, "the state would land in the other buffer");
 
 // Strips of a row: one if the row has no more packs than a warp has lanes (its lanes are then
 // each other's periodic neighbours and nothing is recomputed), else of kUse packs. Warps per
