@@ -41,30 +41,6 @@ constexpr int kUse = 30;
 static_assert(kLevels <= kNV, "wrong nodes would reach the lanes that are stored");
 static_assert(kLevels % 2 == 1, "the state would land in the other buffer");
 
-// Strips of a row: one if the row has no more packs than a warp has lanes (its lanes are then
-// each other's periodic neighbours and nothing is recomputed), else of kUse packs. Warps per
-// block, on neighbouring strips of the same rows: two in FP32 unless that leaves a good part of
-// them idle (4096^2 204 k MLUPS with two, 201 k with one), one in 16-bit storage (8192^2 227 k
-// with one, 221 k with two).
-struct Strips {
-    int packs, warps, groups, segs;
-    Strips(int storage, int nx, int ny, int64_t resident_warps) {
-        packs = nx / kNV;
-        const int strips = packs <= 32 ? 1 : (packs + kUse - 1) / kUse;
-        warps = storage == kStoreF32 && (strips % 2 == 0 || strips > 8) ? 2 : 1;
-        groups = (strips + warps - 1) / warps;
-        // One segment of rows per resident block and strip group. Segments under 8 rows repeat
-        // too many relaxations (2 (kLevels - 1) rows each): half as many then (FP32 1536 x 1000
-        // 145 k MLUPS against 138 k). Long 16-bit segments are halved, so that blocks that end
-        // early leave work to take (8192^2 227 k against 224 k; no gain in FP32).
-        int64_t s = resident_warps / warps / groups;
-        if (s * 8 > ny) s = resident_warps / 2 / warps / groups;
-        if (storage != kStoreF32 && s * 64 < ny) s = 2 * s;
-        if (s > ny) s = ny;
-        segs = (int)(s < 1 ? 1 : s);
-    }
-};
-
 // A pack in storage form: NV consecutive nodes in W 32-bit words.
 template <typename T>
 constexpr int kW = kNV * (int)sizeof(T) / 4;
@@ -180,6 +156,44 @@ constexpr int kSmem = kSlot<T, WPB> * 9 * kLevels + (UM == UM_FIELD ? 2 * 32 * W
 // levels stay in registers.
 template <int UM>
 constexpr int kSmWarps = UM == UM_FIELD ? 12 : 16;
+
+// Warps that an SM holds in blocks of `warps` warps: by its registers, and by its 228 KB of
+// shared memory, of which every block takes 1 KB more than it asks for (FP32 blocks of one warp:
+// 15). Sized for 16, the grid left a last wave, or, at half of it, blocks that did not fit beside
+// those of the launch before (u~ = q/rho, us a step, sized for 16 -> 15: 600 x 4000 17.5 -> 15.1,
+// 800 x 1000 10.9 -> 7.1, 64 x 9000 12.8 -> 7.4).
+int sm_warps(int storage, int um, int warps) {
+    const int slot = 32 * warps * kNV * (storage == kStoreF32 ? 4 : 2);
+    const int smem = slot * 9 * kLevels + (um == UM_FIELD ? 2 * 32 * warps * 16 : 0);
+    const int by_regs = (um == UM_FIELD ? kSmWarps<UM_FIELD> : kSmWarps<UM_ZERO>) / warps;
+    const int by_smem = 228 * 1024 / (smem + 1024);
+    return (by_regs < by_smem ? by_regs : by_smem) * warps;
+}
+
+// Strips of a row: one if the row has no more packs than a warp has lanes (its lanes are then
+// each other's periodic neighbours and nothing is recomputed), else of kUse packs. Warps per
+// block, on neighbouring strips of the same rows: two in FP32 unless that leaves a good part of
+// them idle (4096^2 204 k MLUPS with two, 201 k with one), one in 16-bit storage (8192^2 227 k
+// with one, 221 k with two).
+struct Strips {
+    int packs, warps, groups, segs;
+    Strips(int storage, int um, int nx, int ny) {
+        packs = nx / kNV;
+        const int strips = packs <= 32 ? 1 : (packs + kUse - 1) / kUse;
+        warps = storage == kStoreF32 && (strips % 2 == 0 || strips > 8) ? 2 : 1;
+        groups = (strips + warps - 1) / warps;
+        const int64_t resident_warps = (int64_t)sm_warps(storage, um, warps) * sm_count();
+        // One segment of rows per resident block and strip group. Segments under 8 rows repeat
+        // too many relaxations (2 (kLevels - 1) rows each): half as many then (FP32 1536 x 1000
+        // 145 k MLUPS against 138 k). Long 16-bit segments are halved, so that blocks that end
+        // early leave work to take (8192^2 227 k against 224 k; no gain in FP32).
+        int64_t s = resident_warps / warps / groups;
+        if (s * 8 > ny) s = resident_warps / 2 / warps / groups;
+        if (storage != kStoreF32 && s * 64 < ny) s = 2 * s;
+        if (s > ny) s = ny;
+        segs = (int)(s < 1 ? 1 : s);
+    }
+};
 
 template <typename T, int UM, int BASIS, int RCP, int WPB>
 __global__ void __launch_bounds__(32 * WPB, kSmWarps<UM> / WPB)
@@ -332,8 +346,7 @@ cudaError_t launch_w(const void* src, void* dst, const StepArgs& a, const MarchA
 template <typename T, int UM, int BASIS, int RCP>
 cudaError_t launch_t(const void* src, void* dst, const StepArgs& a, const MarchAmps& amps,
                      cudaStream_t st) {
-    const Strips p(sizeof(T) == 4 ? kStoreF32 : kStoreF16, a.nx, a.ny,
-                   (int64_t)kSmWarps<UM> * sm_count());
+    const Strips p(sizeof(T) == 4 ? kStoreF32 : kStoreF16, UM, a.nx, a.ny);
     if constexpr (sizeof(T) == 4) {
         if (p.warps == 2) return launch_w<T, UM, BASIS, RCP, 2>(src, dst, a, amps, p, st);
     }
@@ -391,8 +404,8 @@ double march_step_us(int storage, int um, int basis, int nx, int ny, const void*
         return kNoForm;
     // Measured on GB300: 0.235 nodes per ns and lane in use with every warp resident, 0.205
     // with half of them, 6 rows repeated in three per segment, a third of a launch.
-    const int64_t warps = (int64_t)(um == UM_FIELD ? 12 : 16) * sm_count();
-    const Strips p(storage, nx, ny, warps);
+    const Strips p(storage, um, nx, ny);
+    const int64_t warps = (int64_t)sm_warps(storage, um, p.warps) * sm_count();
     const double useful = (double)p.packs / (32.0 * p.groups * p.warps);
     const double rows = (double)ny / p.segs;
     const bool half = (int64_t)p.groups * p.warps * p.segs * 3 < warps * 2;
