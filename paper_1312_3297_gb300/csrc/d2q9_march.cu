@@ -162,11 +162,12 @@ constexpr int kSmWarps = UM == UM_FIELD ? 12 : 16;
 // 15). Sized for 16, the grid left a last wave, or, at half of it, blocks that did not fit beside
 // those of the launch before (u~ = q/rho, us a step, sized for 16 -> 15: 600 x 4000 17.5 -> 15.1,
 // 800 x 1000 10.9 -> 7.1, 64 x 9000 12.8 -> 7.4).
+constexpr int kSmSmem = 228 * 1024, kSmemMost = 227 * 1024;
 int sm_warps(int storage, int um, int warps) {
     const int slot = 32 * warps * kNV * (storage == kStoreF32 ? 4 : 2);
     const int smem = slot * 9 * kLevels + (um == UM_FIELD ? 2 * 32 * warps * 16 : 0);
     const int by_regs = (um == UM_FIELD ? kSmWarps<UM_FIELD> : kSmWarps<UM_ZERO>) / warps;
-    const int by_smem = 228 * 1024 / (smem + 1024);
+    const int by_smem = kSmSmem / (smem + 1024);
     return (by_regs < by_smem ? by_regs : by_smem) * warps;
 }
 
@@ -335,10 +336,21 @@ cudaError_t launch_w(const void* src, void* dst, const StepArgs& a, const MarchA
     constexpr int smem = kSmem<T, UM, WPB>;
     static std::atomic<int> resident[kMaxDevicesOcc];  // sets the kernel's shared memory, once
     int full = 0;
-    cudaError_t e = resident_blocks(kernel, resident, 32 * WPB, smem, 32, &full);
+    cudaError_t e = resident_blocks(kernel, resident, 32 * WPB, kSmemMost, 32, &full);
     if (e != cudaSuccess) return e;
-    e = launch_pdl_smem(kernel, dim3((unsigned)((int64_t)p.groups * p.segs)), dim3(32 * WPB), smem,
-                        st, static_cast<const T*>(src), static_cast<T*>(dst), a, amps, p.groups,
+    const int64_t blocks = (int64_t)p.groups * p.segs;
+    // Blocks of a dependent launch start on whatever SM its predecessor has left, several on
+    // one and none on another, and the launch after that fills the gaps they leave. So where an
+    // SM would hold more than its share, ask for as much shared memory as lets just that fit.
+    const int64_t share = (blocks + sm_count() - 1) / sm_count();
+    int smem = kSmem<T, UM, WPB>;
+    if (share * WPB < sm_warps(sizeof(T) == 4 ? kStoreF32 : kStoreF16, UM, WPB)) {
+        const int only = ((int)(kSmSmem / share) - 1024) / 128 * 128;  // allocated by 128 bytes
+        if (smem < only) smem = only;
+        if (smem > kSmemMost) smem = kSmemMost;
+    }
+    e = launch_pdl_smem(kernel, dim3((unsigned)blocks), dim3(32 * WPB), smem, st,
+                        static_cast<const T*>(src), static_cast<T*>(dst), a, amps, p.groups,
                         p.segs);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
