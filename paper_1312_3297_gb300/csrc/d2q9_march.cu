@@ -333,7 +333,6 @@ template <typename T, int UM, int BASIS, int RCP, int WPB>
 cudaError_t launch_w(const void* src, void* dst, const StepArgs& a, const MarchAmps& amps,
                      const Strips& p, cudaStream_t st) {
     auto kernel = k_march3<T, UM, BASIS, RCP, WPB>;
-    constexpr int smem = kSmem<T, UM, WPB>;
     static std::atomic<int> resident[kMaxDevicesOcc];  // sets the kernel's shared memory, once
     int full = 0;
     cudaError_t e = resident_blocks(kernel, resident, 32 * WPB, kSmemMost, 32, &full);
