@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <cmath>
 
 #include "async_copy.cuh"
 #include "d2q9.cuh"
@@ -413,19 +414,25 @@ double march_step_us(int storage, int um, int basis, int nx, int ny, const void*
     if (um == UM_FIELD && (reinterpret_cast<uintptr_t>(ut0) % 16 != 0 ||
                            (storage != kStoreF32 && basis == 1 && nx % 8 != 0)))
         return kNoForm;
-    // Measured on GB300: 0.235 nodes per ns and lane in use with every warp resident, 0.205
-    // with half of them, 6 rows repeated in three per segment, a third of a launch.
+    // Fitted as single_step_us is: a launch; the rows that a warp marches through, with a latency
+    // of their own or, beside enough other warps, the SM's share; the memory beyond L2.
     const Strips p(storage, um, nx, ny);
-    const int64_t warps = (int64_t)sm_warps(storage, um, p.warps) * sm_count();
-    const double useful = (double)p.packs / (32.0 * p.groups * p.warps);
-    const double rows = (double)ny / p.segs;
-    const bool half = (int64_t)p.groups * p.warps * p.segs * 3 < warps * 2;
-    // the correctly rounded 1/rho is slower, the more so with few warps to hide it
-    const bool rn = um != UM_ZERO && (storage == kStoreF32 ? basis == 1
-                                                           : basis == 0 && nx % 8 != 0);
-    const double rate = (half ? 205.0 : 235.0) * (um == UM_FIELD ? 0.82 : 1.0) *
-                        (!rn ? 1.0 : half && storage != kStoreF32 ? 0.7 : 0.9);
-    return (double)nx * ny / (rate * 1e3 * useful) * (1.0 + 2.0 / rows) + 0.7;
+    const bool f32 = storage == kStoreF32, field = um == UM_FIELD;
+    const double rows = (ny + p.segs - 1) / p.segs + 2 * (kLevels - 1);
+    const double warps = (double)p.groups * p.warps * p.segs / sm_count();  // per SM
+    const int most = sm_warps(storage, um, p.warps);
+    const double busy = std::ceil(warps < most ? warps : most);
+    const double latency = f32 ? (field ? 0.954 : 0.786) : (field ? 0.917 : 0.953);
+    const double share = (f32 ? (field ? 0.256 : 0.170) : (field ? 0.253 : 0.196)) * busy;
+    constexpr double modes[2][2][4] = {{{1.0, 1.21, 1.22, 1.0}, {1.28, 1.46, 1.52, 1.24}},
+                                       {{1.0, 0.97, 1.0, 1.0}, {1.04, 0.98, 1.01, 1.01}}};
+    const double l2 = latency * latency, s2 = share * share;
+    double row = modes[!f32][basis][um] * std::sqrt(std::sqrt(l2 * l2 + s2 * s2));
+    if (!f32 && basis == 0 && um != UM_ZERO && nx % 8 != 0) row *= 1.24;  // 1/rho correctly rounded
+    const double us = 1.2 + rows * row * (warps > most ? warps / most : 1.0) +
+                      (field ? 0.0 : f32 ? 1.12 : 2.2) * 1e-6 * ((double)nx * ny) *
+                          beyond_l2(storage, um, nx, ny, 40e6, 130e6);
+    return us / kLevels * (beyond_l2(storage, um, nx, ny, 125e6, 125e6) > 0.0 ? 0.9 : 1.0);
 }
 
 cudaError_t launch_march(int storage, int um, const void* src, void* dst, const StepArgs& a,

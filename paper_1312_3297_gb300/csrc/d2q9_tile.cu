@@ -5,19 +5,36 @@ namespace lbmrv {
 
 namespace {
 
-// Times in microseconds measured on GB300, for the choice of a plan only (any plan gives the
-// same states).
-constexpr double kLaunch = 2.1;      // a pass: launch, first loads, last stores
+// The models below choose between forms and plans only (any choice gives the same states). Their
+// numbers are fitted to single steps, three-step passes and tile launches of 10,500 random
+// lattices of 8 - 4300 nodes a side, all storages, modes and bases, timed on GB300 (microseconds);
+// each predicts these to 7 % (standard deviation).
 constexpr double kStepFloor = 0.46;  // a step of a block that fills no pipe
 constexpr double kItem = 0.0545;     // a warp's two rows of 32 nodes on a busy SM, per SM
 constexpr double kSerial = 2.0;      // loads and stores of a tile that nothing else overlaps
 
 bool fits_l2(double nodes, int node_bytes) { return 2.0 * node_bytes * nodes < 128e6; }
 
-// the correctly rounded 1/rho of 16-bit storage, and the conversions, take a little longer
-double tile_item_us(int elem, int um, int nv) {
-    return kItem * (elem == 2 && um != UM_ZERO ? (nv == 8 ? 1.03 : 1.1) : 1.0);
-}
+// A pass's fixed part and, relative to the numbers above, its steps: by storage, basis and mode,
+// and by the relaxation that the pack width decides (node by node, or with the correctly rounded
+// 1/rho).
+struct TileCost {
+    double launch, scale;
+    TileCost(int storage, int um, int basis, int nv) {
+        constexpr double fixed[4] = {1.85, 1.8, 2.1, 2.35};
+        constexpr double steps[2][2][4] = {{{0.88, 1.06, 1.20, 1.09}, {1.00, 1.17, 1.24, 1.13}},
+                                           {{0.94, 1.11, 1.23, 1.08}, {1.00, 1.13, 1.21, 1.12}}};
+        const bool half = storage != kStoreF32;
+        launch = fixed[um];
+        scale = steps[half][basis][um];
+        if (half && basis == 1 && (nv <= 2 || (nv == 4 && um == UM_FIELD))) {
+            launch += 0.2;
+            scale *= 1.12;
+        } else if (half && basis == 0 && um != UM_ZERO && nv < 8) {
+            scale *= 1.02;
+        }
+    }
+};
 
 }  // namespace
 
@@ -35,45 +52,73 @@ int sm_count() {
     return sms;
 }
 
-// The launch, and the time per million nodes at the pack width nv: with the states in L2, too
-// large for it, or between; more where a row leaves many of a block's 128 threads without a
-// pack.
-double single_step_us(int storage, int um, int nv, int nx, int ny) {
-    const double nodes = (double)nx * ny;
-    const bool f32 = storage == kStoreF32;
-    const double field = um == UM_FIELD ? 8.0 : 0.0;
-    const double both = (2.0 * 9.0 * (f32 ? 4 : 2) + field) * nodes;
-    const bool l2 = both < 78e6, dram = both > 128e6;
-    double per_m;
-    if (f32)
-        per_m = nv == 4 ? (l2 ? 6.4 : dram ? 10.5 : 7.8)
-              : nv == 2 ? (dram ? 10.9 : 8.2)
-                        : (dram ? 11.2 : 7.7);
+// A launch; its blocks, warps and nodes (in L2, and beyond it); and, for blocks between half and
+// all of those resident at once, the blocks of the next launch, which start early, leaving some
+// SMs with more of them than others (FP32 1016 x 352, 704 blocks: 6.8 us where 528 take 3).
+double single_step_us(int storage, int um, int basis, int nv, int nx, int ny) {
+    struct Row {
+        double launch, block, warp, l2, dram, pile;
+        double mode[8];  // u~ = 0, 0 in Geier's basis, q/rho, ...
+    };
+    constexpr Row f32[3] = {
+        {1.52, 0.34, 0.07, 3.74, 7.25, 1.23, {1.0, 1.07, 1.11, 1.17, 1.28, 1.27, 1.27, 1.26}},
+        {1.82, 0.60, 0.21, 1.05, 5.39, 1.96, {1.0, 0.92, 1.27, 1.08, 0.99, 1.13, 1.23, 1.14}},
+        {1.94, 0.63, 0.24, 2.17, 6.77, 2.75, {1.0, 1.11, 1.16, 1.20, 1.19, 1.32, 1.21, 1.28}}};
+    constexpr Row half[4] = {
+        {1.53, 0.22, 0.12, 2.75, 3.91, 1.01, {1.0, 1.23, 1.25, 1.32, 1.44, 1.41, 1.34, 1.38}},
+        {1.69, 0.60, 0.17, 1.01, 1.93, 1.73, {1.0, 1.07, 1.18, 1.17, 1.25, 1.26, 1.24, 1.25}},
+        {1.93, 0.63, 0.30, 0.57, 2.16, 0.89, {1.0, 1.02, 1.22, 1.19, 1.31, 1.27, 1.42, 1.38}},
+        {2.16, 1.22, 0.56, 0.72, 2.15, 0.93, {1.0, 1.03, 1.04, 1.09, 1.08, 1.20, 1.23, 1.29}}};
+    const bool is_f32 = storage == kStoreF32;
+    const int i = nv == 8 ? 3 : nv == 4 ? 2 : nv - 1;
+    const Row& c = is_f32 ? f32[i] : half[i];
+    const int threads = nv == 1 ? 256 : 128, packs = nx / nv;
+    const double blocks = (double)((packs + threads - 1) / threads) * ny;
+    const double warps = (double)((packs + 31) / 32) * ny;
+    // blocks per SM, by the kernels' registers
+    int per_sm;
+    if (nv == 1)
+        per_sm = 6;
+    else if (nv == 2)
+        per_sm = 8;
+    else if (nv == 8)
+        per_sm = basis ? (um == UM_FIELD ? 4 : 5) : um <= UM_FLUID ? 4 : 3;
+    else if (is_f32)
+        per_sm = um <= UM_FLUID ? 7 : 6;
     else
-        per_m = nv == 8 ? (dram ? 5.8 : 4.4) : nv == 4 ? 5.4 : nv == 2 ? 7.7 : 9.5;
-    if (nv >= 4) {
-        const int span = 128 * nv;
-        const double used = (double)nx / (span * ((nx + span - 1) / span));
-        if (f32)
-            per_m *= used < 0.1 ? 0.3 / used : 1.0 + 0.2 * (1.0 - used);
-        else
-            per_m *= used < 0.4 ? 0.5 / used : 1.0 + 0.8 * (1.0 - used);
+        per_sm = basis == 1 && um != UM_FIELD ? 8 : 6;
+    const double share = blocks / (per_sm * sm_count());
+    double pile = 1.0;
+    if (share > 0.56 && share < 1.0) {
+        const double busy = (warps / blocks - 1.0) / (threads / 32 - 1);  // warps of a block
+        pile += c.pile * (1.0 - share) * (busy < 1.0 ? busy : 1.0);
     }
-    if (um == UM_ZERO && !f32 && !dram) per_m *= 0.87;
-    if (um == UM_FIELD) per_m *= !dram || f32 ? 1.07 : 1.22;
-    return 1.9 + per_m * 1e-6 * nodes;
+    const double m = (double)nx * ny * 1e-6, far = beyond_l2(storage, um, nx, ny, 78e6, 135e6);
+    return c.launch + pile * (c.mode[2 * um + basis] * (c.block * blocks * 1e-3 +
+                                                        c.warp * warps * 1e-3 +
+                                                        c.l2 * m * (1.0 - far)) +
+                              c.dram * m * far);
+}
+
+// 0 if both states and a stored field take less than lo bytes, 1 if more than hi.
+double beyond_l2(int storage, int um, int nx, int ny, double lo, double hi) {
+    const double bytes = ((storage == kStoreF32 ? 72.0 : 36.0) + (um == UM_FIELD ? 8.0 : 0.0)) *
+                         ((double)nx * ny);
+    return bytes <= lo ? 0.0 : bytes >= hi ? 1.0 : (bytes - lo) / (hi - lo);
 }
 
 namespace {
 
 // The array and warps per block that take a launch of s steps in the least modelled time
 // (steps = 1 if that is `least` or more).
-TilePlan tile_pass(int storage, int um, int nv, int nx, int ny, int s, double least) {
+TilePlan tile_pass(int storage, int um, int basis, int nv, int nx, int ny, int s,
+                   double least) {
     TilePlan best;
     best.us = least;
     const int elem = storage == kStoreF32 ? 4 : 2, sms = sm_count();
     const bool in_l2 = fits_l2((double)nx * ny, 9 * elem);
-    const double item_us = tile_item_us(elem, um, nv);
+    const TileCost cost(storage, um, basis, nv);
+    const double item_us = kItem * cost.scale, floor_us = kStepFloor * cost.scale;
     const double per_sm = item_us / sms;
     // the first step's loads: latency that few later steps leave exposed
     const double first = (s == 2 ? (in_l2 ? 1.5 : 2.0) : s == 3 ? 1.2 : 1.0) +
@@ -91,8 +136,8 @@ TilePlan tile_pass(int storage, int um, int nv, int nx, int ny, int s, double le
             const int tiles = tiles_x * ((ny + ty - 1) / ty);
             // the pipes' share, were the tiles spread evenly: usually enough to drop it
             const double even = per_sm * s * (rx / 32) * ((ry + ty) / 4) * tiles;
-            const double steps_alone = kStepFloor * s;
-            if (kLaunch + (even > steps_alone ? even : steps_alone) >= best.us) continue;
+            const double steps_alone = floor_us * s;
+            if (cost.launch + (even > steps_alone ? even : steps_alone) >= best.us) continue;
             const int items = rx / 32 * (ry / 2);
             const int rounds = (items + kTileWarps - 1) / kTileWarps;
             const int whole = (items + rounds - 1) / rounds;
@@ -113,17 +158,16 @@ TilePlan tile_pass(int storage, int um, int nv, int nx, int ny, int s, double le
                         const int pairs = rx / 32 * ((ry - k - 1) / 2 - k / 2 + 1);
                         const double pipes = (k ? 1.0 : first) * item * pairs * resident;
                         const double alone =
-                            pairs <= warps ? kStepFloor
-                                           : kStepFloor * ((pairs + warps - 1) / warps);
+                            pairs <= warps ? floor_us : floor_us * ((pairs + warps - 1) / warps);
                         us += pipes > alone ? pipes : alone;
                     }
                     return us;
                 };
                 const int full = tiles / (sms * fit), rest = tiles - full * sms * fit;
                 double us = full * wave(fit) + (rest ? wave((rest + sms - 1) / sms) : 0.0);
-                if (fit == 1 && tiles > sms) us += kSerial * (tiles - sms) / sms;
-                if (kLaunch + us < best.us) {
-                    best.us = kLaunch + us;
+                if (fit == 1 && tiles > sms) us += kSerial * cost.scale * (tiles - sms) / sms;
+                if (cost.launch + us < best.us) {
+                    best.us = cost.launch + us;
                     best.steps = s;
                     best.rx = rx;
                     best.ry = ry;
@@ -148,15 +192,15 @@ TilePlan tile_pass(int storage, int um, int nv, int nx, int ny, int s, double le
 // Measured, single steps -> here, us a step (u~ = q/rho): FP32 64^2 2.05 -> 0.82, 256^2 2.3 ->
 // 1.22, 512^2 3.9 -> 2.73, 1023^2 10.1 -> 8.3, 4097 x 1999 94 -> 60; FP16 64^2 2.1 -> 0.87,
 // 512^2 3.0 -> 2.9, 513 x 511 4.5 -> 2.9, 4097 x 1999 82 -> 60.
-TilePlan tile_plan(TileTable& table, int storage, int um, int nv, int nx, int ny, int64_t n,
-                   double least) {
+TilePlan tile_plan(TileTable& table, int storage, int um, int basis, int nv, int nx, int ny,
+                   int64_t n, double least) {
     TilePlan best;
     best.us = least;
     // What a launch of s steps takes at least: the launch, and each step's latency or the pipes'
     // share of the lattice.
-    const double share = tile_item_us(storage == kStoreF32 ? 4 : 2, um, nv) * (double)nx * ny /
-                         (64.0 * sm_count());
-    const double step = share > kStepFloor ? share : kStepFloor;
+    const TileCost cost(storage, um, basis, nv);
+    const double share = kItem * (double)nx * ny / (64.0 * sm_count());
+    const double step = cost.scale * (share > kStepFloor ? share : kStepFloor);
     // likely lengths first: a good plan early drops most of the others unsearched
     constexpr int lengths[] = {5, 10, 4, 3, 8, 6, 12, 2};
     for (int want : lengths) {
@@ -165,11 +209,11 @@ TilePlan tile_plan(TileTable& table, int storage, int um, int nv, int nx, int ny
         int64_t m = (n + want - 1) / want;
         m += (m ^ n) & 1;
         const int s = (int)((n + m - 1) / m);
-        if (s < 2 || m * (kLaunch + step * s) >= best.us) continue;
+        if (s < 2 || m * (cost.launch + step * s) >= best.us) continue;
         TilePlan& pass = table.best[s];
         const double least = best.us / m;
         if (pass.steps == 1 && pass.us < least)
-            pass = tile_pass(storage, um, nv, nx, ny, s, least);
+            pass = tile_pass(storage, um, basis, nv, nx, ny, s, least);
         if (pass.steps > 1 && pass.us < least) {
             best = pass;
             best.us = m * pass.us;

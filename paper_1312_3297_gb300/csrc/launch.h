@@ -39,7 +39,8 @@ int sm_count();
 // step: one launch per step at pack width nv; one of launch_march's three (kNoForm where it does
 // not suit the lattice: row length, alignment; ut0 the stored field, or null).
 constexpr double kNoForm = 1e30;
-double single_step_us(int storage, int um, int nv, int nx, int ny);
+double single_step_us(int storage, int um, int basis, int nv, int nx, int ny);
+double beyond_l2(int storage, int um, int nx, int ny, double lo, double hi);
 double march_step_us(int storage, int um, int basis, int nx, int ny, const void* a,
                      const void* b, const float* ut0);
 
@@ -55,7 +56,6 @@ cudaError_t launch_march(int storage, int um, const void* src, void* dst, const 
 // p.steps steps src -> dst in one launch on shared-memory tiles (d2q9_tile.cuh): arrays of p.rx
 // x p.ry nodes, blocks of p.warps warps. The bits of that many launch_step calls at pack width nv.
 constexpr int kTileMaxSteps = 12;
-constexpr int kTileMinSteps = 5;  // of a call: fewer steps are left to the other forms
 constexpr int kTileMaxSmem = 224 * 1024;
 constexpr int kTileWarps = 24;  // most per block and per SM
 struct TileAmps {
@@ -79,8 +79,8 @@ inline int64_t tile_bytes(int rx, int ry, int elem, int um) {
            (um == UM_FIELD ? 8LL * rx * (ry + 1) : um == UM_ANALYTIC ? 4LL * (ry + 1) : 0);
 }
 // Plan of n steps; steps = 1 unless it takes less than `least` microseconds.
-TilePlan tile_plan(TileTable& table, int storage, int um, int nv, int nx, int ny, int64_t n,
-                   double least);
+TilePlan tile_plan(TileTable& table, int storage, int um, int basis, int nv, int nx, int ny,
+                   int64_t n, double least);
 cudaError_t launch_tile(int storage, int um, int basis, int nv, const void* src, void* dst,
                         const StepArgs& a, const TileAmps& amps, const TilePlan& p,
                         cudaStream_t st);

@@ -132,3 +132,37 @@ def test_plan_follows_the_width_and_the_count():
     assert sim.step_plan(20)[0] == "tile"
     sim.set_kernel_width(4)
     assert sim.step_plan(20) == ("single", 20, 1, 0)
+
+
+# lattices whose states fit L2 or nearly do, where the forms' times cross
+CROSSING = [("D2Q9Cascaded", 1560, 656, "fp32", "field", 7),
+            ("D2Q9Cascaded", 928, 1528, "fp32", "prescribed", 7),
+            ("D2Q9Cascaded", 352, 2369, "fp32", "zero", 10),
+            ("D2Q9Cascaded", 2024, 734, "fp32", "prescribed", 10),
+            ("D2Q9", 160, 1136, "fp16", "fluid", 4),
+            ("D2Q9", 528, 1504, "fp32", "prescribed", 4),
+            ("D2Q9", 352, 1464, "fp32", "field", 100)]
+
+
+@pytest.mark.parametrize("lattice,nx,ny,storage,mode,n", CROSSING)
+def test_the_chosen_form_is_not_slower_than_single_steps(lattice, nx, ny, storage, mode, n):
+    """Calls of n steps back to back, in turn with single steps, best of several series; the
+    margin is for what is left of the models' error (two series differ by under 2 %)."""
+    import torch
+
+    one, auto = _pair(lattice, nx, ny, mode, storage, "auto")
+    calls = max(4, 200 // n)
+    best = {}
+    for _ in range(6):
+        for sim in (one, auto):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            sim.step(n)
+            torch.cuda.synchronize()
+            torch.cuda._sleep(200000)
+            a.record(sim.stream)
+            for _ in range(calls):
+                sim.step(n)
+            b.record(sim.stream)
+            b.synchronize()
+            best[sim] = min(best.get(sim, float("inf")), a.elapsed_time(b))
+    assert best[auto] <= 1.15 * best[one]
