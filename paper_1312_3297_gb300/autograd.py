@@ -2,8 +2,8 @@
 
 ``Rollout.apply(u0, s_nu, amp, sim, n, seg, rho0)`` sets the state of ``sim`` to the
 equilibrium of (rho0, u0), advances n steps with checkpoints every ``seg`` steps, and returns
-the final density and velocity fields. With ``seg`` None or 0 the checkpoints are as dense as a
-sixteenth of the free memory allows, see ``default_workspace``; the gradient does not depend on
+the final density and velocity fields. With ``seg`` None or 0 the checkpoints are as dense as
+the free memory allows, see ``default_workspace``; the gradient does not depend on
 the interval, bit for bit. The backward pass runs the hand-written
 discrete adjoint of the library (moments adjoint, reverse sweep, equilibrium adjoint),
 giving gradients with respect to the initial velocity field, the shear rate s_nu (the
@@ -19,8 +19,12 @@ import weakref
 import torch
 
 
-# Share of a device's memory that checkpoints may take without being asked for.
+# Shares of a device's memory that checkpoints may take without being asked for: one rollout's,
+# of all memory; what those of all live rollouts hold beyond sqrt(n) checkpoints, of the free
+# memory; and what needs no look at the free memory (the look takes 9 us).
 CHECKPOINT_SHARE = 1 / 16
+LIVE_SHARE = 1 / 8
+SMALL_SHARE = 1 / 1024
 
 # Bytes that the workspaces alive on each device hold beyond those of sqrt(n) checkpoints.
 _extra: dict = {}
@@ -48,21 +52,27 @@ def _give_back(device, nbytes: int):
 
 
 def default_workspace(sim, n: int):
-    """Checkpoint interval and workspace of a rollout that names no interval. What it holds
-    beyond sqrt(n) checkpoints, together with what all others alive on the device hold beyond
-    theirs, stays within CHECKPOINT_SHARE of the memory that the driver would have free with
-    sqrt(n) checkpoints only: a program that keeps many rollouts alive, or that leaves little memory free, gets
-    sqrt(n) checkpoints, as it does where the allocation fails."""
+    """Checkpoint interval and workspace of a rollout that names no interval. The workspace takes
+    at most CHECKPOINT_SHARE of the device's memory, unless sqrt(n) checkpoints need more. What
+    it holds beyond those, together with what all others alive on the device hold beyond
+    theirs, stays within LIVE_SHARE of the memory that the driver would have free with sqrt(n)
+    checkpoints only: a program that keeps many rollouts alive, or that leaves little memory
+    free, gets sqrt(n) checkpoints, as it does where the allocation fails."""
     longest = max(1, math.ceil(math.sqrt(n)))
-    least = sim.adjoint_workspace_bytes(n, longest)
-    device = str(sim.device)
+    if longest == 1:
+        return 1, sim.adjoint_workspace(n, 1)
+    device = sim.device
+    least, most = (sim.adjoint_workspace_bytes(n, seg) for seg in (longest, 1))
+    total = torch.cuda.get_device_properties(device).total_memory
     with _extra_lock:
         held = _extra.setdefault(device, 0)
-        room = 0.0
-        if longest > 1:
-            spare = torch.cuda.mem_get_info(sim.device)[0] + held - least
-            room = CHECKPOINT_SHARE * max(0, spare) - held
-        seg = checkpoint_interval(sim, n, least + room)
+        if held + most - least <= SMALL_SHARE * total:
+            seg = 1
+        else:
+            index = device.index if device.index is not None else torch.cuda.current_device()
+            free = torch.cuda.cudart().cudaMemGetInfo(index)[0]
+            room = LIVE_SHARE * max(0, free + held - least) - held
+            seg = checkpoint_interval(sim, n, min(least + room, CHECKPOINT_SHARE * total))
         more = max(0, sim.adjoint_workspace_bytes(n, seg) - least)
         _extra[device] += more
     try:

@@ -1,6 +1,7 @@
 """Memory of rollouts that name no checkpoint interval."""
 import gc
 import math
+import types
 
 import pytest
 
@@ -13,7 +14,7 @@ N = 200
 class _Sim:
     """Workspace sizes of a 1024^2 lattice; the workspaces themselves are small."""
 
-    device = "cuda:0"
+    device = torch.device("cuda", 0)
 
     def __init__(self, device_memory):
         self.memory = device_memory
@@ -56,9 +57,16 @@ def autograd(monkeypatch):
     return module
 
 
+TOTAL = 280 << 30
+
+
 def _use(monkeypatch, memory):
-    monkeypatch.setattr(torch.cuda, "mem_get_info", lambda d: (
-        memory.told if memory.told is not None else memory.free, 1 << 60))
+    def info(index):
+        return (memory.told if memory.told is not None else memory.free), TOTAL
+
+    monkeypatch.setattr(torch.cuda, "cudart", lambda: types.SimpleNamespace(cudaMemGetInfo=info))
+    monkeypatch.setattr(torch.cuda, "get_device_properties",
+                        lambda d: types.SimpleNamespace(total_memory=TOTAL))
     return _Sim(memory)
 
 
@@ -66,23 +74,37 @@ LONGEST = math.ceil(math.sqrt(N))
 
 
 def test_many_live_rollouts_together_stay_within_the_share(monkeypatch, autograd):
-    """As many rollouts as fit with sqrt(n) checkpoints and a sixteenth of the memory spare:
-    every one is served, and together they hold no more than that sixteenth beyond what sqrt(n)
+    """As many rollouts as fit with sqrt(n) checkpoints and an eighth of the memory spare: every
+    one is served, and together they hold no more than that eighth beyond what sqrt(n)
     checkpoints hold."""
-    total = 280 << 30
-    memory = _Memory(total)
+    memory = _Memory(TOTAL)
     sim = _use(monkeypatch, memory)
     least = sim.adjoint_workspace_bytes(N, LONGEST)
-    count = int(total * (1 - autograd.CHECKPOINT_SHARE) / least)
+    count = int(TOTAL * (1 - autograd.LIVE_SHARE) / least)
     live = []
     for k in range(count):
         live.append(autograd.default_workspace(sim, N))
-        assert total - memory.free <= (k + 1) * least + autograd.CHECKPOINT_SHARE * total
-    assert live[0][0] == 1 and live[-1][0] > 1
+        assert TOTAL - memory.free <= (k + 1) * least + autograd.LIVE_SHARE * TOTAL
+    assert live[2][0] == 1 and live[-1][0] > 1
     del live
     gc.collect()
-    assert memory.free == total and autograd._extra == {"cuda:0": 0}
+    assert memory.free == TOTAL and autograd._extra == {sim.device: 0}
     assert autograd.default_workspace(sim, N)[0] == 1  # given back
+
+
+def test_one_rollout_stays_within_its_share(monkeypatch, autograd):
+    sim = _use(monkeypatch, _Memory(TOTAL))
+    n = 4000
+    seg, ws = autograd.default_workspace(sim, n)
+    assert 1 < seg < math.ceil(math.sqrt(n))
+    assert sim.adjoint_workspace_bytes(n, seg) <= autograd.CHECKPOINT_SHARE * TOTAL
+    assert sim.adjoint_workspace_bytes(n, seg - 1) > autograd.CHECKPOINT_SHARE * TOTAL
+
+
+def test_small_workspaces_need_no_look_at_the_memory(monkeypatch, autograd):
+    sim = _use(monkeypatch, _Memory(TOTAL))
+    monkeypatch.setattr(torch.cuda, "cudart", None)
+    assert autograd.default_workspace(sim, 9)[0] == 1
 
 
 def test_little_free_memory_means_least_memory(monkeypatch, autograd):
@@ -96,20 +118,19 @@ def test_little_free_memory_means_least_memory(monkeypatch, autograd):
 def test_a_failed_allocation_falls_back(monkeypatch, autograd):
     """The driver reports free memory that the allocation then does not get."""
     memory = _Memory(2 << 30)
-    memory.told = 280 << 30
-    seg, ws = autograd.default_workspace(_use(monkeypatch, memory), N)
-    assert seg == LONGEST and autograd._extra == {"cuda:0": 0}
+    memory.told = TOTAL
+    sim = _use(monkeypatch, memory)
+    seg, ws = autograd.default_workspace(sim, N)
+    assert seg == LONGEST and autograd._extra == {sim.device: 0}
 
 
-def test_one_step_needs_no_question(monkeypatch, autograd):
+def test_one_step(monkeypatch, autograd):
     sim = _use(monkeypatch, _Memory(1 << 30))
-    monkeypatch.setattr(torch.cuda, "mem_get_info", None)
-    assert autograd.default_workspace(sim, 1)[0] == 1
+    assert autograd.default_workspace(sim, 1)[0] == 1 and autograd._extra == {}
 
 
 def test_invalid_windows_are_refused(monkeypatch, autograd):
-    memory = _Memory(280 << 30)
-    sim = _use(monkeypatch, memory)
+    sim = _use(monkeypatch, _Memory(TOTAL))
     monkeypatch.setattr(_Sim, "adjoint_workspace_bytes", lambda self, n, seg: -1)
 
     def refuse(self, n, seg):
@@ -118,7 +139,7 @@ def test_invalid_windows_are_refused(monkeypatch, autograd):
     monkeypatch.setattr(_Sim, "adjoint_workspace", refuse)
     with pytest.raises(ValueError):
         autograd.default_workspace(sim, N)
-    assert autograd._extra == {"cuda:0": 0}
+    assert autograd._extra == {sim.device: 0}
 
 
 @pytest.mark.gpu
