@@ -332,37 +332,47 @@ __global__ void __launch_bounds__(32 * WPB, kSmWarps<UM> / WPB)
 
 template <typename T, int UM, int BASIS, int RCP, int WPB>
 cudaError_t launch_w(const void* src, void* dst, const StepArgs& a, const MarchAmps& amps,
-                     const Strips& p, cudaStream_t st) {
+                     const Strips& p, cudaStream_t st, MarchStart start) {
     auto kernel = k_march3<T, UM, BASIS, RCP, WPB>;
     static std::atomic<int> resident[kMaxDevicesOcc];  // sets the kernel's shared memory, once
     int full = 0;
     cudaError_t e = resident_blocks(kernel, resident, 32 * WPB, kSmemMost, 32, &full);
     if (e != cudaSuccess) return e;
-    const int64_t blocks = (int64_t)p.groups * p.segs;
     // Blocks of a dependent launch start on whatever SM its predecessor has left, several on
-    // one and none on another, and the launch after that fills the gaps they leave. So where an
-    // SM would hold more than its share, ask for as much shared memory as lets just that fit.
+    // one and none on another, and the launch after that fills the gaps they leave: with single
+    // steps before them, the passes of a whole call ran up to 1.4 times longer. So of a few
+    // passes each asks for as much shared memory as lets an SM hold its share of the blocks and
+    // no more (BF16 816 x 2096, calls of 10 steps, us a step, 14.6 -> 10.9), and of many the first
+    // starts alone, which spreads the blocks evenly, and the others follow freely (stored field,
+    // FP32 1536 x 1000, 50 steps: 1.4 % faster than each with its share).
+    const int64_t blocks = (int64_t)p.groups * p.segs;
     const int64_t share = (blocks + sm_count() - 1) / sm_count();
     int smem = kSmem<T, UM, WPB>;
-    if (share * WPB < sm_warps(sizeof(T) == 4 ? kStoreF32 : kStoreF16, UM, WPB)) {
+    if (start == MarchStart::kShare &&
+        share * WPB < sm_warps(sizeof(T) == 4 ? kStoreF32 : kStoreF16, UM, WPB)) {
         const int only = ((int)(kSmSmem / share) - 1024) / 128 * 128;  // allocated by 128 bytes
         if (smem < only) smem = only;
         if (smem > kSmemMost) smem = kSmemMost;
     }
-    e = launch_pdl_smem(kernel, dim3((unsigned)blocks), dim3(32 * WPB), smem, st,
-                        static_cast<const T*>(src), static_cast<T*>(dst), a, amps, p.groups,
-                        p.segs);
+    const T* const from = static_cast<const T*>(src);
+    T* const to = static_cast<T*>(dst);
+    const dim3 grid((unsigned)blocks);
+    if (start == MarchStart::kAlone)
+        kernel<<<grid, 32 * WPB, smem, st>>>(from, to, a, amps, p.groups, p.segs);
+    else
+        e = launch_pdl_smem(kernel, grid, dim3(32 * WPB), smem, st, from, to, a, amps, p.groups,
+                            p.segs);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T, int UM, int BASIS, int RCP>
 cudaError_t launch_t(const void* src, void* dst, const StepArgs& a, const MarchAmps& amps,
-                     cudaStream_t st) {
+                     cudaStream_t st, MarchStart start) {
     const Strips p(sizeof(T) == 4 ? kStoreF32 : kStoreF16, UM, a.nx, a.ny);
     if constexpr (sizeof(T) == 4) {
-        if (p.warps == 2) return launch_w<T, UM, BASIS, RCP, 2>(src, dst, a, amps, p, st);
+        if (p.warps == 2) return launch_w<T, UM, BASIS, RCP, 2>(src, dst, a, amps, p, st, start);
     }
-    return launch_w<T, UM, BASIS, RCP, 1>(src, dst, a, amps, p, st);
+    return launch_w<T, UM, BASIS, RCP, 1>(src, dst, a, amps, p, st, start);
 }
 
 // 1/rho in the form that the one-step kernel of the same rows uses (d2q9_kernels.cu), so that
@@ -371,36 +381,36 @@ cudaError_t launch_t(const void* src, void* dst, const StepArgs& a, const MarchA
 // correctly rounded one.
 template <typename T, int BASIS, int UM>
 cudaError_t launch_rcp(const void* s, void* d, const StepArgs& a, const MarchAmps& amps,
-                       cudaStream_t st) {
+                       cudaStream_t st, MarchStart start) {
     if constexpr (sizeof(T) == 4) {
-        return launch_t<T, UM, BASIS, BASIS == 0 ? RCP_APPROX : RCP_RN>(s, d, a, amps, st);
+        return launch_t<T, UM, BASIS, BASIS == 0 ? RCP_APPROX : RCP_RN>(s, d, a, amps, st, start);
     } else if constexpr (UM == UM_ZERO) {
-        return launch_t<T, UM, BASIS, RCP_RN>(s, d, a, amps, st);
+        return launch_t<T, UM, BASIS, RCP_RN>(s, d, a, amps, st, start);
     } else {
         if constexpr (BASIS == 0) {
-            if (a.nx % 8 != 0) return launch_t<T, UM, BASIS, RCP_RN>(s, d, a, amps, st);
+            if (a.nx % 8 != 0) return launch_t<T, UM, BASIS, RCP_RN>(s, d, a, amps, st, start);
         }
-        return launch_t<T, UM, BASIS, RCP_DIV>(s, d, a, amps, st);
+        return launch_t<T, UM, BASIS, RCP_DIV>(s, d, a, amps, st, start);
     }
 }
 
 template <typename T, int BASIS>
 cudaError_t launch_um(int um, const void* s, void* d, const StepArgs& a, const MarchAmps& amps,
-                      cudaStream_t st) {
+                      cudaStream_t st, MarchStart start) {
     switch (um) {
-        case UM_ZERO: return launch_rcp<T, BASIS, UM_ZERO>(s, d, a, amps, st);
-        case UM_FLUID: return launch_rcp<T, BASIS, UM_FLUID>(s, d, a, amps, st);
-        case UM_ANALYTIC: return launch_rcp<T, BASIS, UM_ANALYTIC>(s, d, a, amps, st);
-        case UM_FIELD: return launch_rcp<T, BASIS, UM_FIELD>(s, d, a, amps, st);
+        case UM_ZERO: return launch_rcp<T, BASIS, UM_ZERO>(s, d, a, amps, st, start);
+        case UM_FLUID: return launch_rcp<T, BASIS, UM_FLUID>(s, d, a, amps, st, start);
+        case UM_ANALYTIC: return launch_rcp<T, BASIS, UM_ANALYTIC>(s, d, a, amps, st, start);
+        case UM_FIELD: return launch_rcp<T, BASIS, UM_FIELD>(s, d, a, amps, st, start);
         default: return cudaErrorInvalidValue;
     }
 }
 
 template <typename T>
 cudaError_t launch_basis(int um, const void* s, void* d, const StepArgs& a,
-                         const MarchAmps& amps, cudaStream_t st, int basis) {
-    return basis == 0 ? launch_um<T, 0>(um, s, d, a, amps, st)
-                      : launch_um<T, 1>(um, s, d, a, amps, st);
+                         const MarchAmps& amps, cudaStream_t st, int basis, MarchStart start) {
+    return basis == 0 ? launch_um<T, 0>(um, s, d, a, amps, st, start)
+                      : launch_um<T, 1>(um, s, d, a, amps, st, start);
 }
 
 }  // namespace
@@ -436,11 +446,11 @@ double march_step_us(int storage, int um, int basis, int nx, int ny, const void*
 }
 
 cudaError_t launch_march(int storage, int um, const void* src, void* dst, const StepArgs& a,
-                         const MarchAmps& amps, cudaStream_t st, int basis) {
+                         const MarchAmps& amps, cudaStream_t st, int basis, MarchStart start) {
     switch (storage) {
-        case kStoreF32: return launch_basis<float>(um, src, dst, a, amps, st, basis);
-        case kStoreF16: return launch_basis<__half>(um, src, dst, a, amps, st, basis);
-        case kStoreBF16: return launch_basis<__nv_bfloat16>(um, src, dst, a, amps, st, basis);
+        case kStoreF32: return launch_basis<float>(um, src, dst, a, amps, st, basis, start);
+        case kStoreF16: return launch_basis<__half>(um, src, dst, a, amps, st, basis, start);
+        case kStoreBF16: return launch_basis<__nv_bfloat16>(um, src, dst, a, amps, st, basis, start);
         default: return cudaErrorInvalidValue;
     }
 }

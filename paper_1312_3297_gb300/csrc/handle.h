@@ -13,6 +13,19 @@
 #include "launch.h"
 #include "lbmrv.h"
 
+namespace lbmrv {
+// How n steps are split into launches: `marches` passes of kMarchSteps steps, or tile.launches
+// passes over tiles, and single steps for the rest; for a mode, form and alignment of the
+// relative-velocity field.
+struct StepPlan {
+    int64_t n = 0;
+    int um = -1, form = 0;
+    bool aligned = false;
+    int64_t marches = 0;
+    TilePlan tile;
+};
+}  // namespace lbmrv
+
 struct lbmrv_s {
     int lattice = LBMRV_D2Q9;
     int q = 9;       // populations per node
@@ -42,6 +55,7 @@ struct lbmrv_s {
     // arrays of the tile kernel found so far: without, with a stored relative-velocity field
     lbmrv::TileTable tiles[2];
     int form = 0;  // LBMRV_FORM_*
+    lbmrv::StepPlan plans[4];  // the last ones made, of n steps in [n % 4]
     double* red = nullptr;   // reduction scratch: 8 * red_blocks partials + 8 results
     int red_blocks = 0;
     double* host = nullptr;  // 8 results that kernels write and the host reads (mapped memory)

@@ -47,11 +47,14 @@ double march_step_us(int storage, int um, int basis, int nx, int ny, const void*
 // kMarchSteps steps src -> dst in one pass over memory (d2q9_march.cu), the bits of that many
 // launch_step calls. a: the arguments of the first of them; amps: amp_t of each.
 constexpr int kMarchSteps = 3;
+constexpr int kMarchMany = 8;  // passes of a call from which on the first of them starts alone
+enum class MarchStart { kShare, kAlone, kFollow };  // see launch_w in d2q9_march.cu
 struct MarchAmps {
     float v[kMarchSteps];
 };
 cudaError_t launch_march(int storage, int um, const void* src, void* dst, const StepArgs& a,
-                         const MarchAmps& amps, cudaStream_t st, int basis);
+                         const MarchAmps& amps, cudaStream_t st, int basis,
+                         MarchStart start);
 
 // p.steps steps src -> dst in one launch on shared-memory tiles (d2q9_tile.cuh): arrays of p.rx
 // x p.ry nodes, blocks of p.warps warps. The bits of that many launch_step calls at pack width nv.

@@ -459,16 +459,9 @@ int lbmrv_init_equilibrium_host(lbmrv_t h, const float* rho_host, const float* u
                             "lbmrv_init_equilibrium_host");
 }
 
-// How n steps are split into launches: `marches` passes of kMarchSteps steps, or tile.launches
-// passes over tiles, and single steps for the rest.
-struct StepPlan {
-    int64_t marches = 0;
-    TilePlan tile;
-};
-static StepPlan plan_steps(lbmrv_t h, int nv, int64_t n) {
+static StepPlan make_plan(lbmrv_t h, int nv, int um, int64_t n) {
     StepPlan p;
-    if (n < 2 || h->dim != 2 || h->width != 0 || h->slab || h->form == LBMRV_FORM_SINGLE) return p;
-    const int nx = (int)h->nx, ny = (int)h->ny, um = kernel_mode(h);
+    const int nx = (int)h->nx, ny = (int)h->ny;
     const int64_t rest = n % kMarchSteps;
     const double march = march_step_us(h->storage, um, h->basis, nx, ny, h->f[0], h->f[1], h->ut0);
     if (h->form == LBMRV_FORM_MARCH) {
@@ -492,6 +485,24 @@ static StepPlan plan_steps(lbmrv_t h, int nv, int64_t n) {
     p.tile = tile_plan(h->tiles[um == UM_FIELD], h->storage, um, h->basis, nv, nx, ny, n,
                        0.98 * (marched < n * step ? marched : n * step));
     if (p.tile.steps == 1 && marched < n * step) p.marches = n / kMarchSteps;
+    return p;
+}
+
+// The plan of n steps. Making it takes 0.3 us where the tile arrays are known, so the last few
+// are kept.
+static StepPlan plan_steps(lbmrv_t h, int nv, int64_t n) {
+    if (n < 2 || h->dim != 2 || h->width != 0 || h->slab || h->form == LBMRV_FORM_SINGLE)
+        return StepPlan();
+    const int um = kernel_mode(h);
+    const bool aligned = reinterpret_cast<uintptr_t>(h->ut0) % 16 == 0;
+    StepPlan& p = h->plans[n % 4];
+    if (p.n != n || p.um != um || p.form != h->form || p.aligned != aligned) {
+        p = make_plan(h, nv, um, n);
+        p.n = n;
+        p.um = um;
+        p.form = h->form;
+        p.aligned = aligned;
+    }
     return p;
 }
 
@@ -539,8 +550,11 @@ int lbmrv_step(lbmrv_t h, int64_t n) {
     for (int64_t m = plan.marches; m > 0; --m, k += kMarchSteps) {
         MarchAmps amps;
         for (int l = 0; l < kMarchSteps; ++l) amps.v[l] = prescribed_amp(h, h->t + 1 + l);
+        const MarchStart start = plan.marches < kMarchMany ? MarchStart::kShare
+                                 : k == 0                  ? MarchStart::kAlone
+                                                           : MarchStart::kFollow;
         cudaError_t e = launch_march(h->storage, um, h->f[h->cur], h->f[1 - h->cur],
-                                     make_args(h, h->t + 1), amps, h->stream, h->basis);
+                                     make_args(h, h->t + 1), amps, h->stream, h->basis, start);
         if (e != cudaSuccess) return cuda_fail(h, e, "lbmrv_step");
         h->cur = 1 - h->cur;
         h->t += kMarchSteps;

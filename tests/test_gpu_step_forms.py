@@ -66,7 +66,7 @@ MARCH = [(4, 90001), (128, 2500), (132, 2500), (1800, 2003), (1804, 2001), (1796
 
 @every
 def test_march(lattice, mode, storage):
-    for sizes, counts in ((MARCH_TINY, (3, 4, 7)), (MARCH, (3, 7))):
+    for sizes, counts in ((MARCH_TINY, (3, 4, 7, 25)), (MARCH, (3, 7, 26))):
         for nx, ny in sizes:
             if (mode, lattice) == ("field", "D2Q9Cascaded") and storage != "fp32" and nx % 8:
                 continue  # refused: see below
