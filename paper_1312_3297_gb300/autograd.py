@@ -14,7 +14,6 @@ from __future__ import annotations
 
 import math
 import threading
-import weakref
 
 import torch
 
@@ -46,9 +45,17 @@ def checkpoint_interval(sim, n: int, budget: float | None = None) -> int:
     return longest
 
 
-def _give_back(device, nbytes: int):
-    with _extra_lock:
-        _extra[device] -= nbytes
+class _Lease:
+    """Bytes of _extra[device], given back when it goes."""
+
+    __slots__ = ("device", "nbytes")
+
+    def __init__(self, device, nbytes: int):
+        self.device, self.nbytes = device, nbytes
+
+    def __del__(self):
+        with _extra_lock:
+            _extra[self.device] -= self.nbytes
 
 
 def default_workspace(sim, n: int):
@@ -72,17 +79,18 @@ def default_workspace(sim, n: int):
             index = device.index if device.index is not None else torch.cuda.current_device()
             free = torch.cuda.cudart().cudaMemGetInfo(index)[0]
             room = LIVE_SHARE * max(0, free + held - least) - held
-            seg = checkpoint_interval(sim, n, min(least + room, CHECKPOINT_SHARE * total))
-        more = max(0, sim.adjoint_workspace_bytes(n, seg) - least)
+            budget = min(least + room, CHECKPOINT_SHARE * total)
+            seg = 1 if most <= budget else checkpoint_interval(sim, n, budget)
+        more = max(0, (most if seg == 1 else sim.adjoint_workspace_bytes(n, seg)) - least)
         _extra[device] += more
+    lease = _Lease(device, more)
     try:
         ws = sim.adjoint_workspace(n, seg)
-    except BaseException as e:
-        _give_back(device, more)
-        if more == 0 or not isinstance(e, torch.cuda.OutOfMemoryError):
+    except torch.cuda.OutOfMemoryError:
+        if more == 0:
             raise
         return longest, sim.adjoint_workspace(n, longest)
-    weakref.finalize(ws, _give_back, device, more)
+    ws.lease = lease  # given back with the workspace, or on the way out
     return seg, ws
 
 

@@ -27,7 +27,7 @@ class _Sim:
         if size > self.memory.free:
             raise torch.cuda.OutOfMemoryError("no room")
         ws = torch.empty(1)
-        ws.lease = self.memory.take(size)
+        ws.memory = self.memory.take(size)
         return ws
 
 
