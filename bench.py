@@ -3,9 +3,11 @@
 Headline workload: D2Q9 FP32, 4096 x 4096 periodic, Taylor-Green vortex u0 = 0.04,
 rho0 = 1, s = (0,0,0,1.4,1.8,1.8,1.2,1.2,1.4) (s_nu = 1.8), prescribed relative velocity
 u~(x,t) = 0.03 (cos 2 pi y/L, sin 2 pi x/L) cos(2 pi t / 1000). One bench step is one
-time step (pull transport + relaxation in the moving frame), one kernel launch. The
-0.6 GB state (1.2 GB moved per step) is larger than L2, so no flush is needed between
-steps.
+time step (pull transport + relaxation in the moving frame); the library takes three steps
+per kernel launch, and the launches reported are those of its own plan of the timed call
+(lbmrv_step_plan). The 0.6 GB state (1.2 GB moved per launch) is larger than L2, so no flush
+is needed between launches. An untimed call of the timed length precedes the warm-up steps:
+CUDA loads a kernel at its first launch, which is not part of a step.
 
 ``python bench.py [--gpus N] [--steps K] [--warmup W]`` prints one JSON line.
 ``--impl reference`` times the FP64 CPU oracle on the host cores instead (same metric).
@@ -33,7 +35,6 @@ L = 4096
 S_RATES = [0, 0, 0, 1.4, 1.8, 1.8, 1.2, 1.2, 1.4]
 UT_AMP, UT_PERIOD = 0.03, 1000.0
 BYTES_PER_NODE = {"fp32": 72, "fp16": 36, "bf16": 36}  # a D2Q9 state read and written once
-STEPS_PER_PASS = 3  # D2Q9 steps per pass over memory, states beyond L2, automatic kernel
 WORKLOAD = ("D2Q9 relative-velocity step, FP32, 4096x4096 periodic, Taylor-Green u0=0.04, "
             "s_nu=1.8, prescribed u~ = 0.03 (cos 2pi y/L, sin 2pi x/L) cos(2pi t/1000)")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "d2q9_step_tg4096_traffic.txt")
@@ -188,15 +189,6 @@ def default_width(lattice: str, storage: str, nx: int) -> int:
     return widest
 
 
-def passes(steps: int, lattice: str = "d2q9", width: int = 0, decomp: str = "replicas") -> int:
-    """Step-kernel launches for `steps` steps of one call on a lattice beyond L2: D2Q9 with the
-    automatic kernel takes three steps per pass over memory, the rest one by one. On smaller
-    lattices the library may take more steps per launch, so there it is an upper bound."""
-    if lattice != "d2q9" or width or decomp == "slab":
-        return steps
-    return steps // STEPS_PER_PASS + steps % STEPS_PER_PASS
-
-
 def bandwidth(nodes: int, bytes_per_pass: float, steps: int, launches: int, ms: float,
               peak: float) -> dict:
     """What `launches` passes moved (each reads and writes the state once), and the same time
@@ -206,15 +198,18 @@ def bandwidth(nodes: int, bytes_per_pass: float, steps: int, launches: int, ms: 
             "frac_at_one_step_per_pass": round(gbs / peak * steps / launches, 4)}
 
 
-def kernel_label(lattice: str, storage: str, nx: int, mode: str, scheme: str = "rv",
-                 width: int = 0) -> str:
-    """Name of the step kernel the library launches for this configuration."""
+def kernel_label(plan: tuple, lattice: str, storage: str, nx: int, mode: str,
+                 scheme: str = "rv", width: int = 0) -> str:
+    """Name of the step kernel that takes most of the steps of a call with this plan
+    (``step_plan`` of the simulation)."""
+    form, launches, longest, _ = plan
     nv = width or default_width(lattice, storage, nx)
-    if lattice == "d2q9" and not width and nx % 4 == 0:
-        basis = "" if scheme == "rv" else ", Geier basis"
-        return f"k_march3<{storage},{mode}{basis}> ({STEPS_PER_PASS} steps per launch)"
+    basis = "" if scheme == "rv" else ", Geier basis"
+    if form in ("march", "tile"):
+        name = "k_march3" if form == "march" else "k_tile"
+        return f"{name}<{storage},{mode}{basis}> ({longest} steps per launch)"
     if lattice == "d2q9":
-        name = "k_step_vec" if scheme == "rv" else "k_step_vec, Geier basis"
+        name = ("k_step_vec" if nv > 1 else "k_step_scalar") + basis
     elif storage == "fp32":
         name = "k_step3"
     else:
@@ -258,14 +253,15 @@ def side_measure(torch, D2Q9, inp, storage, mode, size, fields, steps, peak, u_r
                  stored_field=False):
     sim = make_sim(torch, D2Q9, inp, storage, mode, size, fields, u_ref=u_ref,
                    stored_field=stored_field)
-    sim.step(3)
+    sim.step(steps)
     ms = time_steps(sim, steps, torch)
+    launches = sim.step_plan(steps)[1]
     sim.close()
     n = size * size
     per = ms / steps
     bpn = BYTES_PER_NODE[storage] + (8 if stored_field else 0)  # + the field's two floats
     return {"mlups": round(n / (per * 1e-3) / 1e6, 1), "ms_per_step": round(per, 5),
-            **bandwidth(n, bpn, steps, passes(steps), ms, peak)}
+            **bandwidth(n, bpn, steps, launches, ms, peak)}
 
 
 class SlabRun:
@@ -278,6 +274,9 @@ class SlabRun:
 
     def step(self, n=1):
         self.slab.step(n)
+
+    def step_plan(self, n):
+        return "single", n, 1, 0  # every step exchanges halo rows
 
     def conserved(self, allow_nonfinite=False):
         c = self.slab.conserved3()
@@ -339,6 +338,7 @@ def gpu_arm(args):
         sim = make_sim(torch, scheme, inp, args.storage, args.mode, size, fields)
         if args.width:
             sim.set_kernel_width(args.width)
+    sim.step(args.steps)  # first use of the kernels of such a call
     sim.step(args.warmup)
     torch.cuda.synchronize()
     clocks = ClockSampler(local) if rank == 0 else None
@@ -368,6 +368,7 @@ def gpu_arm(args):
         repeats = {"steps_per_run": k_rep, "ms_per_step_runs": [round(r, 5) for r in runs],
                    "ms_per_step_median": round(statistics.median(runs), 5)}
     finite = sim.conserved(allow_nonfinite=True)
+    plan = sim.step_plan(args.steps)
     sim.close()
     per_step_ms = ms / args.steps
     mlups = job_mlups(n, world, args.steps, ms)
@@ -382,7 +383,7 @@ def gpu_arm(args):
         e2e["value"] = round(job_mlups(n, world, args.steps, worst * 1e3), 1)
         e2e["runs_rank0"] = e2e.pop("runs")
     pass_bytes = BYTES_PER_NODE[args.storage] * (19 / 9 if args.lattice == "d3q19" else 1)
-    launches = passes(args.steps, args.lattice, args.width, args.decomp)
+    launches = plan[1]
     bpn = pass_bytes * launches / args.steps
     achieved = bpn * n / (per_step_ms * 1e-3) / 1e9
     headline = (size == L and args.storage == "fp32" and args.mode == "prescribed"
@@ -439,7 +440,9 @@ def gpu_arm(args):
                        f"{args.lattice}{' cascaded' if args.scheme == 'cascaded' else ''} "
                        f"{args.storage} side {size} Taylor-Green, u~ mode {args.mode}",
                        "nodes": n, "bytes_per_node_step": round(bpn, 1),
-                       "l2": f"state {pass_bytes / 2 * n / 1e9:.2f} GB > 129 MB L2; no flush needed",
+                       "l2": (f"state {pass_bytes / 2 * n / 1e9:.2f} GB > 129 MB L2; no flush needed"
+                              if pass_bytes / 2 * n > 129e6 else
+                              "the states stay in L2 between launches, as in a run"),
                        "parallelism": f"{args.decomp} x{world}"},
             "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak,
                          "unit": "GB/s", "frac": round(achieved / peak, 4),
@@ -448,8 +451,8 @@ def gpu_arm(args):
                          "traffic": recorded_traffic() if headline else None,
                          "peak_kind": peak_kind,
                          "frac_of_nominal_7900": round(achieved / 7900.0, 4),
-                         "kernel": kernel_label(args.lattice, args.storage, size, args.mode,
-                                                args.scheme, args.width)},
+                         "kernel": kernel_label(plan, args.lattice, args.storage, size,
+                                                args.mode, args.scheme, args.width)},
             "clocks": clock_info,
             "e2e": e2e,
             # step kernels of every rank; a slab adds its pack and unpack kernels
@@ -574,12 +577,13 @@ def cascaded_measure(torch, inp, fields, steps, peak):
     sim = D2Q9Cascaded(L, L, [0, 0, 0, 1.3, 1.8, 1.8, 1.5, 1.5, 1.2], mode="fluid")
     sim.init_equilibrium(*(torch.as_tensor(fields[k], dtype=torch.float32)
                            for k in ("rho", "ux", "uy")))
-    sim.step(3)
+    sim.step(steps)
     per = time_steps(sim, steps, torch) / steps
+    launches = sim.step_plan(steps)[1]
     sim.close()
     n = L * L
     return {"mlups": round(n / (per * 1e-3) / 1e6, 1), "ms_per_step": round(per, 5),
-            **bandwidth(n, 72, steps, passes(steps), per * steps, peak)}
+            **bandwidth(n, 72, steps, launches, per * steps, peak)}
 
 
 def cascaded16_measure(torch, big, steps, peak):
@@ -593,11 +597,12 @@ def cascaded16_measure(torch, big, steps, peak):
         sim = D2Q9Cascaded(8192, 8192, S_RATES, mode="fluid", storage=st)
         sim.init_equilibrium(*(torch.as_tensor(big[k], dtype=torch.float32)
                                for k in ("rho", "ux", "uy")))
-        sim.step(3)
+        sim.step(steps)
         per = time_steps(sim, steps, torch) / steps
+        launches = sim.step_plan(steps)[1]
         sim.close()
         out[st] = {"mlups": round(n / (per * 1e-3) / 1e6, 1), "ms_per_step": round(per, 5),
-                   **bandwidth(n, 36, steps, passes(steps), per * steps, peak)}
+                   **bandwidth(n, 36, steps, launches, per * steps, peak)}
     return out
 
 
@@ -777,7 +782,7 @@ def e2e_measure(torch, D2Q9, inp, fields, steps):
     sim = D2Q9(L, L, S_RATES, mode="prescribed", storage="fp32")
     sim.set_utilde(None, UT_AMP, UT_PERIOD)
     sim.init_equilibrium_host(rho_h, u_h)
-    sim.step(3)
+    sim.step(steps)
     sim.moments_host(rho_o, u_o)
     torch.cuda.synchronize()
     runs = []
