@@ -22,6 +22,13 @@ def mode_id(mode) -> int:
     return _MODES[mode] if isinstance(mode, str) else int(mode)
 
 
+# Handle of torch's current stream on a device. torch.cuda.current_stream builds a Stream object
+# on every call (1 us); the direct query is not part of torch's documented interface.
+_current_raw_stream = getattr(
+    torch._C, "_cuda_getCurrentRawStream",
+    lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
 def _in_memory(t: torch.Tensor) -> bool:
     """Whether the tensor's memory holds its values: a lazily negated view (the imaginary part
     of a conjugate) holds their negatives, a symbolic zero nothing."""
@@ -78,9 +85,8 @@ class D2Q9:
 
     # -- stream order between torch's current stream and the handle's stream
     def _on_current_stream(self) -> bool:
-        # by raw handle: torch.cuda.current_stream builds a Stream object on every call
         mine = self.stream if isinstance(self.stream, int) else self.stream.cuda_stream
-        return torch._C._cuda_getCurrentRawStream(self._index) == mine
+        return _current_raw_stream(self._index) == mine
 
     def _sync_in(self):
         """The handle's stream waits for work already queued on torch's current stream
