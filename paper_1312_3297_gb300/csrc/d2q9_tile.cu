@@ -22,8 +22,8 @@ struct TileCost {
     double launch, scale;
     TileCost(int storage, int um, int basis, int nv) {
         constexpr double fixed[4] = {1.85, 1.8, 2.1, 2.35};
-        constexpr double steps[2][2][4] = {{{0.88, 1.06, 1.20, 1.09}, {1.00, 1.17, 1.24, 1.13}},
-                                           {{0.94, 1.11, 1.23, 1.08}, {1.00, 1.13, 1.21, 1.12}}};
+        constexpr double steps[2][2][4] = {{{0.86, 1.04, 1.15, 1.05}, {1.00, 1.16, 1.24, 1.13}},
+                                           {{0.97, 1.11, 1.23, 1.09}, {1.03, 1.12, 1.21, 1.10}}};
         const bool half = storage != kStoreF32;
         launch = fixed[um];
         scale = steps[half][basis][um];

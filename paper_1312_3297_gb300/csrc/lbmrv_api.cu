@@ -474,16 +474,16 @@ static StepPlan make_plan(lbmrv_t h, int nv, int um, int64_t n) {
         return p;
     }
     if (n < kMarchSteps) return p;
-    // The form with the least modelled time, single steps where no other is clearly faster. With
-    // these margins 0.3 % of 11,000 random lattices and counts run more than 1.5 % slower than
-    // single steps, and the best form is missed by 0.5 % on average (with 0.97 for the march,
-    // 1.0 % and the same). A few single steps after the passes cost more than as many among
+    // The form with the least modelled time, the march only where clearly faster than single
+    // steps. With these margins 0.4 % of 22,000 random lattices and counts run more than 1.5 %
+    // slower than single steps, and the best form is missed by 0.3 % on average (with 0.97 for
+    // the march 1 % run slower). A few single steps after the passes cost more than as many among
     // others: the passes' blocks, and theirs, start on SMs that the other kind has left.
     constexpr double change[kMarchSteps] = {0.0, 0.5, 0.25};
     const double step = single_step_us(h->storage, um, h->basis, nv, nx, ny);
     const double marched = (n - rest) * march / 0.9 + (rest + change[rest]) * step;
     p.tile = tile_plan(h->tiles[um == UM_FIELD], h->storage, um, h->basis, nv, nx, ny, n,
-                       0.98 * (marched < n * step ? marched : n * step));
+                       1.02 * (marched < n * step ? marched : n * step));
     if (p.tile.steps == 1 && marched < n * step) p.marches = n / kMarchSteps;
     return p;
 }
