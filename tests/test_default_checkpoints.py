@@ -54,6 +54,7 @@ def autograd(monkeypatch):
 
     gc.collect()
     monkeypatch.setattr(module, "_extra", {})
+    monkeypatch.setattr(module, "_seen", {})
     return module
 
 
@@ -90,6 +91,27 @@ def test_many_live_rollouts_together_stay_within_the_share(monkeypatch, autograd
     gc.collect()
     assert memory.free == TOTAL and autograd._extra == {sim.device: 0}
     assert autograd.default_workspace(sim, N)[0] == 1  # given back
+
+
+def test_the_free_memory_is_looked_at_again(monkeypatch, autograd):
+    """Memory that others took a moment ago is not counted as free, and an allocation that
+    fails makes the next rollout look at once."""
+    sim = _use(monkeypatch, _Memory(TOTAL))
+    clock = [100.0]
+    monkeypatch.setattr(autograd.time, "monotonic", lambda: clock[0])
+    least = sim.adjoint_workspace_bytes(N, LONGEST)
+    assert autograd.default_workspace(sim, N)[0] == 1
+    sim.memory.free = least + (64 << 20)  # taken by others
+    seg, ws = autograd.default_workspace(sim, N)
+    assert sim.adjoint_workspace_bytes(N, seg) == least  # the failed allocation's fallback
+    del ws
+    sim.memory.free = 8 << 30
+    seg, ws = autograd.default_workspace(sim, N)  # fits, but would leave nothing spare
+    assert sim.adjoint_workspace_bytes(N, seg) < least + autograd.LIVE_SHARE * (8 << 30)
+    del ws
+    sim.memory.free = TOTAL
+    clock[0] += 2 * autograd.LOOK_SECONDS
+    assert autograd.default_workspace(sim, N)[0] == 1
 
 
 def test_one_rollout_stays_within_its_share(monkeypatch, autograd):
