@@ -16,8 +16,8 @@
 // ones, three warps per scheduler instead of four, and two or four levels were slower (FP32
 // 4096^2: 150 k MLUPS with two levels, 203 k with four). Steps per pass are odd so that every
 // state lands in the buffer in which as many single steps would leave it.
-// Measured, MLUPS, u~ = q/rho, one step per launch -> here: FP32 3072^2 95 k -> 204 k, 2048^2
-// 91 k -> 177 k; FP16 8192^2 184 k -> 215 k, 2048^2 164 k -> 173 k; BF16 8192^2 185 k -> 227 k.
+// Measured, MLUPS, u~ = q/rho, one step per launch -> here: FP32 3072^2 96 k -> 203 k, 2048^2
+// 91 k -> 176 k; FP16 8192^2 184 k -> 216 k, 2048^2 166 k -> 172 k; BF16 8192^2 185 k -> 228 k.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -344,12 +344,14 @@ cudaError_t launch_w(const void* src, void* dst, const StepArgs& a, const MarchA
     // passes each asks for as much shared memory as lets an SM hold its share of the blocks and
     // no more (BF16 816 x 2096, calls of 10 steps, us a step, 14.6 -> 10.9), and of many the first
     // starts alone, which spreads the blocks evenly, and the others follow freely (stored field,
-    // FP32 1536 x 1000, 50 steps: 1.4 % faster than each with its share).
+    // FP32 1536 x 1000, 50 steps: 1.4 % faster than each with its share). Grids that fill the SMs
+    // need neither (4096^2, calls of 24 steps, the first alone: 0.7 % slower).
     const int64_t blocks = (int64_t)p.groups * p.segs;
     const int64_t share = (blocks + sm_count() - 1) / sm_count();
+    const bool fills =
+        share * WPB >= sm_warps(sizeof(T) == 4 ? kStoreF32 : kStoreF16, UM, WPB);
     int smem = kSmem<T, UM, WPB>;
-    if (start == MarchStart::kShare &&
-        share * WPB < sm_warps(sizeof(T) == 4 ? kStoreF32 : kStoreF16, UM, WPB)) {
+    if (start == MarchStart::kShare && !fills) {
         const int only = ((int)(kSmSmem / share) - 1024) / 128 * 128;  // allocated by 128 bytes
         if (smem < only) smem = only;
         if (smem > kSmemMost) smem = kSmemMost;
@@ -357,7 +359,7 @@ cudaError_t launch_w(const void* src, void* dst, const StepArgs& a, const MarchA
     const T* const from = static_cast<const T*>(src);
     T* const to = static_cast<T*>(dst);
     const dim3 grid((unsigned)blocks);
-    if (start == MarchStart::kAlone)
+    if (start == MarchStart::kAlone && !fills)
         kernel<<<grid, 32 * WPB, smem, st>>>(from, to, a, amps, p.groups, p.segs);
     else
         e = launch_pdl_smem(kernel, grid, dim3(32 * WPB), smem, st, from, to, a, amps, p.groups,
@@ -450,7 +452,8 @@ cudaError_t launch_march(int storage, int um, const void* src, void* dst, const 
     switch (storage) {
         case kStoreF32: return launch_basis<float>(um, src, dst, a, amps, st, basis, start);
         case kStoreF16: return launch_basis<__half>(um, src, dst, a, amps, st, basis, start);
-        case kStoreBF16: return launch_basis<__nv_bfloat16>(um, src, dst, a, amps, st, basis, start);
+        case kStoreBF16:
+            return launch_basis<__nv_bfloat16>(um, src, dst, a, amps, st, basis, start);
         default: return cudaErrorInvalidValue;
     }
 }

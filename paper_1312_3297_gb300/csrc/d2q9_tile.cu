@@ -187,11 +187,11 @@ TilePlan tile_pass(int storage, int um, int basis, int nv, int nx, int ny, int s
 // block. Small lattices take many steps per pass (64^2: 10, over 32 x 22 arrays), since a launch
 // costs as much as four steps; larger ones the array whose tiles just fill the SMs (512^2: 4 over
 // 64 x 38). Aligned rows of larger L2-resident lattices stay with single steps, which the
-// repeated relaxations of the halos would not beat (FP32 1024^2 8.5 us a step against 9.4,
-// 16-bit 768^2 5.0 against 5.6); there is no such limit for rows without vector packs.
-// Measured, single steps -> here, us a step (u~ = q/rho): FP32 64^2 2.05 -> 0.82, 256^2 2.3 ->
-// 1.22, 512^2 3.9 -> 2.73, 1023^2 10.1 -> 8.3, 4097 x 1999 94 -> 60; FP16 64^2 2.1 -> 0.87,
-// 512^2 3.0 -> 2.9, 513 x 511 4.5 -> 2.9, 4097 x 1999 82 -> 60.
+// repeated relaxations of the halos do not beat (FP32 1024^2 8.5 us a step against 8.3, 16-bit
+// 768^2 4.9 against 5.3, 1024^2 6.4 against 8.9); there is no such limit for rows without vector
+// packs. Measured, single steps -> here, us a step (u~ = q/rho, calls of 24 steps): FP32 64^2
+// 2.07 -> 0.81, 256^2 2.3 -> 1.24, 512^2 3.5 -> 2.68, 1023^2 10.0 -> 8.3, 4097 x 1999 93 -> 64;
+// FP16 64^2 2.1 -> 0.87, 512^2 3.0 -> 2.9, 513 x 511 4.5 -> 2.9, 4097 x 1999 82 -> 60.
 TilePlan tile_plan(TileTable& table, int storage, int um, int basis, int nv, int nx, int ny,
                    int64_t n, double least) {
     TilePlan best;

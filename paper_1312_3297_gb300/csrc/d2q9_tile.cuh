@@ -63,7 +63,9 @@ __device__ __forceinline__ int wrap(int v, int n) {
 // array of RX x ry nodes, which every node reads and writes in the same places: odd steps read
 // population j at slot j of the node and leave the result in slot opp(j) of the node; even
 // steps read population j from slot opp(j) of node x - c_j and leave the result in slot j of
-// node x + c_j. So one barrier per step is enough and no second array is needed.
+// node x + c_j. So one barrier per step is enough and no second array is needed. (The "AA" access
+// pattern of P. Bailey et al., Accelerating lattice Boltzmann fluid flow simulations using
+// graphics processors, ICPP 2009, here within a block.)
 // A thread has one column and relaxes two nodes, (x, y) and (x, y + 1), at a time. Rows of
 // the array are RX values per population, populations side by side, so that every shared
 // address is one register plus a constant. Rows -1, ry and ry + 1 of the array are only read for
