@@ -59,8 +59,9 @@ class _Lease:
         self.device, self.nbytes = device, nbytes
 
     def __del__(self):
-        with _extra_lock:
-            _extra[self.device] -= self.nbytes
+        if _extra_lock is not None:  # else the interpreter is going down
+            with _extra_lock:
+                _extra[self.device] -= self.nbytes
 
 
 def default_workspace(sim, n: int):
