@@ -29,10 +29,14 @@ _current_raw_stream = getattr(
     lambda index: torch.cuda.current_stream(index).cuda_stream)
 
 
-def _in_memory(t: torch.Tensor) -> bool:
-    """Whether the tensor's memory holds its values: a lazily negated view (the imaginary part
-    of a conjugate) holds their negatives, a symbolic zero nothing."""
-    return not (t.is_neg() or t._is_zerotensor())
+def _readable_in_place(components) -> bool:
+    """Whether fields of one shape hold their values in their memory: a lazily negated view (the
+    imaginary part of a conjugate) holds the negatives, a symbolic zero nothing."""
+    shape = components[0].shape
+    for c in components:
+        if c.shape != shape or c.is_neg() or c._is_zerotensor():
+            return False
+    return True
 
 
 def storage_id(storage) -> int:
@@ -168,7 +172,7 @@ class D2Q9:
             raise ValueError(f"expected {self.DIM} velocity components")
         rho = torch.as_tensor(rho, dtype=torch.float32, device=self.device).contiguous()
         u = [torch.as_tensor(c, dtype=torch.float32, device=self.device) for c in u_components]
-        if self._on_current_stream() and all(c.shape == u[0].shape and _in_memory(c) for c in u):
+        if self._on_current_stream() and _readable_in_place(u):
             u = [c.contiguous() for c in u]
             B.lbmrv_init_equilibrium_fields(self.h, rho, *u)
         else:  # read on another stream: a copy that the caller's tensors do not share
@@ -195,7 +199,7 @@ class D2Q9:
         B.lbmrv_moments(self.h, rho, u)
         self._sync_out()
         # separate views: unbind's outputs refuse in-place operations under autograd
-        return (rho,) + tuple(u[a] for a in range(self.DIM))
+        return (rho, *[u.select(0, a) for a in range(self.DIM)])
 
     def moments_host(self, rho_host=None, u_host=None):
         if rho_host is None:
